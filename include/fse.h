@@ -254,8 +254,10 @@ int fse_fit_batch_host(fse_ctx *ctx, const void *pix, int64_t npix_total, int dt
 /* fse_fit_batch for a RAGGED batch (stamps of different sizes, 1 to
  * FSE_MAX_PIX pixels, in any order).  The stamps are bucketed on the device
  * into seven size classes (h*w up to 16^2, 24^2, 32^2, 48^2, 64^2, 96^2,
- * 128^2), and each class runs in its own pair of persistent launches whose
- * shared-memory tile fits that class, largest class first.  Results are those of
+ * 128^2), and each class runs in its own three persistent launches whose
+ * shared-memory tile fits that class, the classes side by side: the largest on
+ * `stream`, the others on streams of the context that wait for the
+ * classification and that `stream` waits for.  Results are those of
  * fse_fit_batch, stamp by stamp.  opts->max_pix is not used (each class sets
  * its own); opts->warps_per_cta, if non-zero, applies to every class, else
  * the class uses the choice of fse_autotune or the library default.  With
@@ -448,9 +450,9 @@ int fse_sync_check(fse_ctx *ctx, void *stream);
  * that owns all device memory.  Same arguments, layout and results as
  * fse_fit_batch, on the CURRENT CUDA device; all pointers but opts and err are
  * device pointers owned by the caller.
- *  - Scratch: a file-scope device array of two 32-bit words (the work counter
- *    and the error word), cleared by a cudaMemsetAsync on `stream` before each
- *    launch.  count is limited to 2^31 - 1 stamps, the range the counter
+ *  - Scratch: a file-scope device array of four 32-bit words (a work counter
+ *    per launch and the error word), cleared by a cudaMemsetAsync on `stream`
+ *    before the first launch.  count is limited to 2^31 - 1 stamps, the range the counter
  *    indexes; a larger count returns FSE_EINVAL with a message.
  *  - First call on a device: builds the b(n) table (a kernel and a device
  *    synchronise) and looks up the scratch address; make it before any stream

@@ -38,7 +38,7 @@ static_assert(chunk_units_total() == 64, "the chunks must cover the batch in 64t
 struct fse_ctx {
     int device = 0;
     char err[512] = {0};
-    unsigned int* d_queue = nullptr;   // kQueues work counters
+    unsigned int* d_queue = nullptr;   // kQueues slots of kQueueWords work counters
     unsigned int* d_err = nullptr;     // sticky error word written by the kernels
     unsigned next_queue = 0;
     cudaStream_t aux_stream = nullptr; // second compute stream of the host-buffer pipeline
@@ -56,10 +56,15 @@ struct fse_ctx {
     float* d_ivar = nullptr;
     size_t ivar_cap = 0;
     // ragged path: stamps grouped by size class, and the class bookkeeping
-    // (counts[K] | range[2K] | cursor[K] | work counters[K])
+    // (counts[K] | range[2K] | cursor[K] | work counters[K kQueueWords])
     int32_t* d_perm = nullptr;
     size_t perm_cap = 0;
     unsigned int* d_cls = nullptr;
+    // one stream per size class but the largest, which runs on the call's own
+    // stream; fork: classification done; join[k]: class k done
+    cudaStream_t cls_stream[fse::kClasses - 1] = {};
+    cudaEvent_t cls_fork = nullptr;
+    cudaEvent_t cls_join[fse::kClasses - 1] = {};
     // grow-only per-stamp coefficients of fse_moment_vjp, and growth-curve
     // records of fse_moment_vjp / _jvp
     fse::VjpCoef* d_vjp = nullptr;
@@ -79,7 +84,8 @@ struct fse_ctx {
 
 namespace {
 
-constexpr int kQueues = 64;
+constexpr int kQueues = 64;                        // calls in flight on one context
+constexpr int kQueueWords = fse::kStageQueues;     // work counters of one call
 std::mutex g_table_mutex;
 // the context in which each device's b(n) table was built (0: not built); a
 // device reset makes a new primary context, whose table is built again
@@ -242,10 +248,15 @@ int prepare(fse_ctx* ctx, const void* pix, int dtype, const float* scale, const 
     return FSE_OK;
 }
 
+// The work counters of the next call, in rotation over the kQueues slots.
+unsigned int* next_queue(fse_ctx* ctx) {
+    return ctx->d_queue + static_cast<size_t>(ctx->next_queue++ % kQueues) * kQueueWords;
+}
+
 int run(fse_ctx* ctx, fse::LaunchArgs& a, cudaStream_t stream) {
     if (a.count == 0) return FSE_OK;
-    a.queue = ctx->d_queue + (ctx->next_queue++ % kQueues);
-    cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), stream);
+    a.queue = next_queue(ctx);
+    cudaError_t e = cudaMemsetAsync(a.queue, 0, kQueueWords * sizeof(unsigned int), stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "work counter reset");
     e = fse::launch_estimator(a, stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "estimator launch");
@@ -282,12 +293,28 @@ int grow(fse_ctx* ctx, T** p, size_t* cap, size_t n) {
 
 // ---------------------------------------------------------------- ragged path
 constexpr int kK = fse::kClasses;
+constexpr int kClsWords = (4 + kQueueWords) * kK;   // d_cls
 
 int ragged_workspace(fse_ctx* ctx, int64_t count) {
     int rc = grow(ctx, &ctx->d_perm, &ctx->perm_cap, static_cast<size_t>(count));
     if (rc) return rc;
+    if (!ctx->cls_fork) {
+        // first ragged call: the class streams and their events; kept on failure
+        // and completed by the next call
+        cudaError_t e = cudaSuccess;
+        for (int k = 0; k < kK - 1 && e == cudaSuccess; ++k) {
+            if (!ctx->cls_stream[k]) e = cudaStreamCreateWithFlags(&ctx->cls_stream[k], cudaStreamNonBlocking);
+            if (e == cudaSuccess && !ctx->cls_join[k])
+                e = cudaEventCreateWithFlags(&ctx->cls_join[k], cudaEventDisableTiming);
+        }
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->cls_fork, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return cuda_fail(ctx, e, "ragged streams");
+        }
+    }
     if (!ctx->d_cls) {
-        cudaError_t e = cudaMalloc(&ctx->d_cls, 5 * kK * sizeof(unsigned int));
+        cudaError_t e = cudaMalloc(&ctx->d_cls, kClsWords * sizeof(unsigned int));
         if (e != cudaSuccess) {
             cudaGetLastError();
             return set_error(ctx, FSE_ENOMEM, "ragged workspace: %s", cudaGetErrorString(e));
@@ -313,28 +340,47 @@ void class_shape(const fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o
     launch_shape(o, fse::kClassPix[k], fse::kStageAll, wpc, nw);
 }
 
-// Classification, then the chain's launch pair per size class (largest first),
-// each with a shared-memory tile for its class.  Everything is stream-ordered
-// on `s` with no host synchronisation, so the sequence can be captured.
+// Classification, then the chain's three launches per size class, each with a
+// shared-memory tile for its class.  The classes are independent and run side
+// by side: the largest on `s`, the others on streams of the context that wait
+// for the classification and that `s` waits for.  Each persistent launch ends
+// in a tail of its slowest stamps (a moment launch's last 0.1 ms runs at a
+// tenth of its warps); one class after another pays 21 such tails in a row,
+// side by side one class's tail is filled by the others' stamps.
+// Event-ordered throughout, with no host synchronisation, so the sequence can
+// be captured.
 int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cudaStream_t s) {
     unsigned int* counts = ctx->d_cls;
     unsigned int* range = counts + kK;
     unsigned int* cursor = range + 2 * kK;
     unsigned int* queues = cursor + kK;
-    cudaError_t e = cudaMemsetAsync(counts, 0, kK * sizeof(unsigned int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(queues, 0, kK * sizeof(unsigned int), s);
+    cudaError_t e = cudaMemsetAsync(ctx->d_cls, 0, kClsWords * sizeof(unsigned int), s);
     if (e == cudaSuccess) e = fse::classify_stamps(a.idx, a.count, counts, range, cursor, ctx->d_perm, s);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->cls_fork, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "size classification");
-    for (int k = kK - 1; k >= 0; --k) {
+    int forked = kK - 1;   // classes forked .. kK - 2 have work on their streams
+    for (int k = kK - 1; k >= 0 && e == cudaSuccess; --k) {
+        const cudaStream_t ks = k == kK - 1 ? s : ctx->cls_stream[k];
+        if (k < kK - 1) {
+            e = cudaStreamWaitEvent(ks, ctx->cls_fork, 0);
+            if (e != cudaSuccess) break;
+            forked = k;
+        }
         fse::LaunchArgs b = a;
         b.opts.max_pix = fse::kClassPix[k];
         b.perm = ctx->d_perm;
         b.range = range + 2 * k;
-        b.queue = queues + k;
+        b.queue = queues + k * kQueueWords;
         class_shape(ctx, a, o, k, &b.warps_per_cta, &b.warps_per_stamp);
-        e = fse::launch_estimator(b, s);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "size-class launch");
+        e = fse::launch_estimator(b, ks);
     }
+    // join what was forked, also after an error: the caller's buffers are in use
+    for (int k = kK - 2; k >= forked; --k) {
+        cudaError_t j = cudaEventRecord(ctx->cls_join[k], ctx->cls_stream[k]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, ctx->cls_join[k], 0);
+        if (e == cudaSuccess) e = j;
+    }
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "size-class launch");
     return FSE_OK;
 }
 
@@ -371,10 +417,10 @@ void make_key(const fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, R
 // cannot allocate device memory at the point of the call: a service that must
 // keep its footprint fixed after start-up, code running under a caching
 // allocator that owns all of the device memory, or a caller that holds no
-// fse_ctx.  The estimator's only per-call scratch is the work counter of the
-// persistent launch and the error word of its bounded waits; for those callers
+// fse_ctx.  The estimator's only per-call scratch is the work counters of the
+// persistent launches and the error word of its bounded waits; for those callers
 // both live in this file-scope array instead of in a context's device memory.
-constexpr int kStaticWords = 2;                      // [0] work counter, [1] error word
+constexpr int kStaticWords = kQueueWords + 1;        // the work counters, then the error word
 constexpr int64_t kStaticMaxCount = 0x7fffffffLL;    // the 32-bit counter indexes at most this
 static __device__ __align__(256) unsigned int g_static_scratch[kStaticWords];
 unsigned int* g_static_addr[256];                    // its address on each device
@@ -420,7 +466,7 @@ int fse_create(fse_ctx** out, int device) {
     ctx->device = device;
     DeviceGuard g(device);
     if (!g.ok) { delete ctx; return FSE_ECUDA; }
-    if (cudaMalloc(&ctx->d_queue, kQueues * sizeof(unsigned int)) != cudaSuccess ||
+    if (cudaMalloc(&ctx->d_queue, kQueues * kQueueWords * sizeof(unsigned int)) != cudaSuccess ||
         cudaMalloc(&ctx->d_err, sizeof(unsigned int)) != cudaSuccess) {
         cudaGetLastError();
         fse_destroy(ctx);
@@ -470,6 +516,11 @@ void fse_destroy(fse_ctx* ctx) {
         cudaFree(ctx->d_cls);
         cudaFree(ctx->d_vjp);
         cudaFree(ctx->d_r50);
+        for (int k = 0; k < fse::kClasses - 1; ++k) {
+            if (ctx->cls_stream[k]) cudaStreamDestroy(ctx->cls_stream[k]);
+            if (ctx->cls_join[k]) cudaEventDestroy(ctx->cls_join[k]);
+        }
+        if (ctx->cls_fork) cudaEventDestroy(ctx->cls_fork);
         if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
         if (ctx->aux_stream) cudaStreamDestroy(ctx->aux_stream);
         if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
@@ -758,10 +809,10 @@ int fse_autotune(fse_ctx* ctx, const void* pix, int dtype, const float* scale,
                 b.opts.max_pix = fse::kClassPix[k];
                 b.perm = ctx->d_perm;
                 b.range = range + 2 * k;
-                b.queue = queues + k;
+                b.queue = queues + k * kQueueWords;
                 b.warps_per_cta = wpc;
                 b.warps_per_stamp = nw;
-                e = cudaMemsetAsync(queues + k, 0, sizeof(unsigned int), s);
+                e = cudaMemsetAsync(b.queue, 0, kQueueWords * sizeof(unsigned int), s);
                 if (e == cudaSuccess) e = cudaEventRecord(ev0, s);
                 if (e == cudaSuccess) e = fse::launch_estimator(b, s);
                 if (e == cudaSuccess) e = cudaEventRecord(ev1, s);
@@ -1036,7 +1087,7 @@ int fse_star_fit(fse_ctx* ctx, const void* pix, int dtype, const float* scale, c
     a.max_pix = o.max_pix > 0 ? o.max_pix : FSE_MAX_PIX;
     a.tol = static_cast<float>(o.tol_sig);
     a.max_iter = o.max_iter_mom;
-    a.queue = ctx->d_queue + (ctx->next_queue++ % kQueues);
+    a.queue = next_queue(ctx);
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "work counter reset");
@@ -1092,7 +1143,7 @@ static int moment_grad(fse_ctx* ctx, bool jvp, const void* pix, int dtype, const
         if (rc) return rc;
         a.r50g = ctx->d_r50;
     }
-    a.queue = ctx->d_queue + (ctx->next_queue++ % kQueues);
+    a.queue = next_queue(ctx);
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "work counter reset");
@@ -1197,7 +1248,7 @@ int fse_sersic_chi2_grad(fse_ctx* ctx, const void* pix, int dtype, const float* 
     a.chi2 = chi2;
     a.dparams = dparams;
     a.dpix = dpix;
-    a.queue = ctx->d_queue + (ctx->next_queue++ % kQueues);
+    a.queue = next_queue(ctx);
     a.bnf = fse::bn_table_f32();
     if (!a.bnf) return set_error(ctx, FSE_ECUDA, "b(n) table address");
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1266,9 +1317,9 @@ int fse_fit_batch_static(const void* pix, int dtype, const float* scale, const f
         scratch = g_static_addr[dev];
     }
     a.queue = scratch;
-    a.err = scratch + 1;
+    a.err = scratch + kQueueWords;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // both words must start at zero: one stream-ordered clear before the launch
+    // every word must start at zero: one stream-ordered clear before the launch
     e = cudaMemsetAsync(scratch, 0, kStaticWords * sizeof(unsigned int), s);
     if (e != cudaSuccess) return fail(cuda_fail(&sink, e, "static scratch clear"));
     e = fse::launch_estimator(a, s);

@@ -42,7 +42,9 @@ struct LaunchArgs {
     int64_t count;
     const float* inv_var;
     fse_result* out;
-    unsigned int* queue;     // persistent-kernel work counter (zeroed before launch)
+    unsigned int* queue;     // kStageQueues work counters, zeroed before the first launch: the
+                             // chain's three launches (and the start-up before fse_centroid's)
+                             // take one each, so nothing clears a counter between them
     unsigned int* err;       // sticky error word (bounded waits that expired)
     DevOpts opts;
     int stage;
@@ -58,6 +60,9 @@ struct LaunchArgs {
     const int32_t* perm;
     const unsigned int* range;
 };
+
+// Work counters of one estimator call (one per launch of the chain).
+constexpr int kStageQueues = 3;
 
 // Size classes of the ragged path: class k holds the stamps with
 // kClassPix[k-1] < h*w <= kClassPix[k] (stamps of invalid size go to class 0,

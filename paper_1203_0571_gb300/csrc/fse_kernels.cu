@@ -2315,25 +2315,23 @@ cudaError_t eval_bn(const double* n, double* b, double* db, int64_t count, cudaS
     return cudaGetLastError();
 }
 
-// The start-up launch before a moment launch on the same stream; the work
-// counter is cleared between the two.
-static cudaError_t launch_startup(const LaunchArgs& a, cudaStream_t stream) {
+// Launches a stage with work counter q of the call's kStageQueues.
+template <int STAGE>
+static cudaError_t launch_queued(const LaunchArgs& a, int q, cudaStream_t stream) {
     LaunchArgs u = a;
-    u.stage = kStageStartup;
-    cudaError_t e = launch_stage<kStageStartup>(u, stream);
-    if (e != cudaSuccess || a.static_assign) return e;
-    return cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), stream);
+    u.stage = STAGE;
+    u.queue = a.queue + (a.static_assign ? 0 : q);
+    return launch_stage<STAGE>(u, stream);
 }
 
 cudaError_t launch_estimator(const LaunchArgs& a, cudaStream_t stream) {
+    cudaError_t e = cudaSuccess;
     switch (a.stage) {
-        case kStageCentroid: {
-            cudaError_t e = launch_startup(a, stream);
-            if (e != cudaSuccess) return e;
-            return launch_stage<kStageCentroid>(a, stream);
-        }
-        case kStageEllipticity: return launch_stage<kStageEllipticity>(a, stream);
-        case kStageFit: return launch_stage<kStageFit>(a, stream);
+        case kStageCentroid:
+            e = launch_queued<kStageStartup>(a, 0, stream);
+            return e != cudaSuccess ? e : launch_queued<kStageCentroid>(a, 1, stream);
+        case kStageEllipticity: return launch_queued<kStageEllipticity>(a, 0, stream);
+        case kStageFit: return launch_queued<kStageFit>(a, 0, stream);
         default: {
             // The whole chain as three persistent launches on the same stream:
             // the start-up, the moment iteration, then the fit of the stamps
@@ -2341,20 +2339,12 @@ cudaError_t launch_estimator(const LaunchArgs& a, cudaStream_t stream) {
             // code (instruction fetch stalls grow with a kernel's code), its
             // registers and its tile; the pixels are read from HBM once per
             // launch.
-            cudaError_t e = launch_startup(a, stream);
+            e = launch_queued<kStageStartup>(a, 0, stream);
+            if (e == cudaSuccess) e = launch_queued<kStageMoments>(a, 1, stream);
             if (e != cudaSuccess) return e;
-            LaunchArgs m = a;
-            m.stage = kStageMoments;
-            e = launch_stage<kStageMoments>(m, stream);
-            if (e != cudaSuccess) return e;
-            if (!a.static_assign) {
-                e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), stream);
-                if (e != cudaSuccess) return e;
-            }
             LaunchArgs f = a;
-            f.stage = kStageFit;
             f.chain_fit = 1;
-            return launch_stage<kStageFit>(f, stream);
+            return launch_queued<kStageFit>(f, 2, stream);
         }
     }
 }
