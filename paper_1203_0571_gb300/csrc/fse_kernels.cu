@@ -122,13 +122,14 @@ struct Grp {
     template <int N>
     __device__ __forceinline__ void allsum(float (&v)[N]) const {
         static_assert(N <= 32, "reduction width");
-        warp_allsum(v);
-        if (NW > 1) {
+        if constexpr (NW == 1) {
+            warp_allsum(v);
+        } else {
+            // each warp's totals go to red straight from the lanes that hold them
+            scatter_sum<N, 16>(v, lane);
+            const int j = scatter_index<N>(lane);
             sync();   // the previous reduction's readers are done with red
-            if (lane == 0) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) red[wi * 32 + i] = v[i];
-            }
+            if (j < N) red[wi * 32 + j] = v[0];
             sync();
 #pragma unroll
             for (int i = 0; i < N; ++i) {
@@ -143,29 +144,22 @@ struct Grp {
     template <int N>
     __device__ __forceinline__ void allsum_df(float (&hi)[N], float (&lo)[N]) const {
         static_assert(2 * N <= 32, "reduction width");
-        warp_allsum_df(hi, lo);
-        if (NW > 1) {
+        if constexpr (NW == 1) {
+            warp_allsum_df(hi, lo);
+        } else {
+            scatter_sum_df<N, 16>(hi, lo, lane);
+            const int j = scatter_index<N>(lane);
             sync();
-            if (lane == 0) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    red[wi * 32 + i] = hi[i];
-                    red[wi * 32 + N + i] = lo[i];
-                }
+            if (j < N) {
+                red[wi * 32 + j] = hi[0];
+                red[wi * 32 + N + j] = lo[0];
             }
             sync();
 #pragma unroll
             for (int i = 0; i < N; ++i) {
                 float h = red[i], l = red[N + i];
 #pragma unroll
-                for (int k = 1; k < NW; ++k) {
-                    const float oh = red[k * 32 + i], ol = red[k * 32 + N + i];
-                    const float sum = h + oh;
-                    const float bb = sum - h;
-                    const float e = (h - (sum - bb)) + (oh - bb);
-                    l = (l + ol) + e;
-                    h = sum;
-                }
+                for (int k = 1; k < NW; ++k) df_merge(h, l, red[k * 32 + i], red[k * 32 + N + i]);
                 hi[i] = h;
                 lo[i] = l;
             }
