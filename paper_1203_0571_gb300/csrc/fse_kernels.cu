@@ -36,13 +36,18 @@ __device__ double2 g_bn[kBnNodes];
 __device__ float2 g_bnf[kBnNodes];
 
 // ------------------------------------------------------------------ PTX
-// 2^x to about one ulp, for the final refinement pass: x = k + f with k an
+// 2^x to about one ulp, for the final refinement passes: x = k + f with k an
 // integer and |f| <= 1/2, 2^f from the Taylor series of exp(f ln 2) to degree 7
-// (truncation below 6e-9 relative), then the exponent raised by k.
+// (truncation below 6e-9 relative), then the exponent raised by k.  k comes
+// from adding and subtracting 1.5 2^23 (round to nearest even, exact for
+// |x| < 2^22) and its integer value from the low bits of that sum, instead of
+// a rounding and a conversion instruction, which issue at a quarter of the
+// rate of an add; out-of-range arguments are selected, not branched on.
+// kNonPos: the caller's x is not above 127.
+template <bool kNonPos = false>
 __device__ __forceinline__ float exp2_acc(float x) {
-    if (!(x >= -126.f)) return 0.f;
-    if (x > 127.f) return INFINITY;
-    const float k = rintf(x);
+    const float z = __fadd_rn(x, 12582912.f);
+    const float k = __fsub_rn(z, 12582912.f);
     const float f = x - k;
     // Horner's scheme (about 1.2 ulp; shorter-chain schemes round the leading
     // terms earlier and lose accuracy)
@@ -54,7 +59,10 @@ __device__ __forceinline__ float exp2_acc(float x) {
     p = fmaf(p, f, 2.4022650695910072e-01f);
     p = fmaf(p, f, 6.931471805599453e-01f);
     p = fmaf(p, f, 1.f);
-    return __int_as_float(__float_as_int(p) + (static_cast<int>(k) << 23));
+    float r = __int_as_float(__float_as_int(p) + (__float_as_int(z) << 23));
+    r = x >= -126.f ? r : 0.f;
+    if (!kNonPos) r = x > 127.f ? INFINITY : r;
+    return r;
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -543,13 +551,12 @@ struct BoxWalk {
 // they were (the last pass that summed them).
 template <int NW, bool FOURTH>
 __device__ __forceinline__ void moment_pass(const float* __restrict__ s, int w, const Box& bx,
-                                            const Grp<NW>& g, const MomState& st,
+                                            const Grp<NW>& g, const MomState& st, float cw,
                                             float (&acc)[11]) {
     const float gg = st.g1 * st.g1 + st.g2 * st.g2;
     const float A = 1.f + gg - 2.f * st.g1;
     const float B = 1.f + gg + 2.f * st.g1;
     const float G4 = 4.f * st.g2;
-    const float cw = -kLog2e / (2.f * st.sw * st.sw);
     constexpr int N = FOURTH ? 11 : 6;
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[i] = 0.f;
@@ -608,13 +615,13 @@ struct Pol {
 
 __device__ __noinline__ Pol shear_polarizability(float Q11, float Q12, float Q22, float F40, float F31,
                                                  float F22, float F13, float F04, float g1, float g2,
-                                                 float sw, float e1, float e2);
+                                                 float c, float iT, float e1, float e2);
 
 // The centroid step <x>/N = k dx (Eqs. 5-6) and the ellipticity step
 // dg = (1-|g_w|^2) (P^SH)^-1 (e^obs - e_w) (Eq. 9) with
 // P^SH = X^SH + dX^SH - e (e^SH + de^SH)^T (Eq. 8, A5, A6, B7, B8), evaluated
 // from the eleven weighted moments.  W' = dW/dR^2 = -c W with c = 1/(2 s_w^2).
-__device__ __forceinline__ MomStep moment_step(const float (&m)[11], const MomState& st,
+__device__ __forceinline__ MomStep moment_step(const float (&m)[11], const MomState& st, float c,
                                                float k_gain, bool ellip, bool matched) {
     MomStep r;
     r.ok = false;
@@ -626,7 +633,6 @@ __device__ __forceinline__ MomStep moment_step(const float (&m)[11], const MomSt
     const float gg = g1 * g1 + g2 * g2;
     const float A = 1.f + gg - 2.f * g1, B = 1.f + gg + 2.f * g1;
     if (!(S0 > 0.f)) return r;
-    const float c = 1.f / (2.f * st.sw * st.sw);
     // Eqs. 5-6 with the fixed gain k (k_gain, or 0.75 where the determined
     // gain below is not usable)
     const float kf = k_gain > 0.f ? k_gain : 0.75f;
@@ -689,7 +695,7 @@ __device__ __forceinline__ MomStep moment_step(const float (&m)[11], const MomSt
     if (!(T > 0.f)) return r;
     const float iT = 1.f / T;
     const float e1 = (Q11 - Q22) * iT, e2 = 2.f * Q12 * iT;
-    const Pol P = shear_polarizability(Q11, Q12, Q22, m[6], m[7], m[8], m[9], m[10], g1, g2, st.sw, e1, e2);
+    const Pol P = shear_polarizability(Q11, Q12, Q22, m[6], m[7], m[8], m[9], m[10], g1, g2, c, iT, e1, e2);
     const float det = P.P11 * P.P22 - P.P12 * P.P21;
     if (!(fabsf(det) > 0.f) || !isfinite(det)) return r;
     const float ew = 2.f / (1.f + gg);
@@ -702,18 +708,16 @@ __device__ __forceinline__ MomStep moment_step(const float (&m)[11], const MomSt
 }
 
 // P^SH = X^SH + dX^SH - e (e^SH + de^SH)^T (Eq. 8 with A5, A6, B7, B8) from the
-// second and fourth weighted moments; W' = dW/dR^2 = -c W with
-// c = 1/(2 s_w^2).  Kept out of line: it is called once per pass from two
+// second and fourth weighted moments, with c = 1/(2 s_w^2) (W' = dW/dR^2 =
+// -c W) and iT = 1/(Q11 + Q22).  Kept out of line: it is called once per pass from two
 // places, and the moment kernel's code size (instruction fetch) matters more
 // than a call; arguments and result travel in registers.
 __device__ __noinline__ Pol shear_polarizability(float Q11, float Q12, float Q22, float F40, float F31,
                                                  float F22, float F13, float F04, float g1, float g2,
-                                                 float sw, float e1, float e2) {
+                                                 float c, float iT, float e1, float e2) {
     const float gg = g1 * g1 + g2 * g2;
     const float A = 1.f + gg - 2.f * g1, B = 1.f + gg + 2.f * g1;
     const float T = Q11 + Q22;
-    const float iT = 1.f / T;
-    const float c = 1.f / (2.f * sw * sw);
     const float ApB = A + B, AmB = A - B;
     const float F31m13 = F31 - F13, F31p13 = F31 + F13;
     // Appendix A: sum f W chi_a psi_b and sum f W theta^2 psi_b
@@ -804,7 +808,7 @@ __device__ float moment_refine(const float* __restrict__ s, int h, int w, const 
                           fmaf(A, e11, fmaf(B, e22, -G4 * e12));
         const float x = R2 * cw;
         const float xl = fmaf(R2, cw, -x) + R2l * cw;
-        const float Wh = exp2_acc(x);
+        const float Wh = exp2_acc<true>(x);
         const float W = fmaf(Wh, xl * static_cast<float>(kLn2), Wh);
         const float I = s[p];
         const float f = I * W, fl = fmaf(I, W, -f);
@@ -867,8 +871,8 @@ __device__ float moment_refine(const float* __restrict__ s, int h, int w, const 
         const float T = Q11 + Q22;
         const float den = T * (1.f + gg);
         const float r1 = n1 / den, r2 = n2 / den;
-        const Pol P = shear_polarizability(Q11, Q12, Q22, F[0], F[1], F[2], F[3], F[4], g1, g2, st.sw,
-                                           (Q11 - Q22) / T, 2.f * Q12 / T);
+        const Pol P = shear_polarizability(Q11, Q12, Q22, F[0], F[1], F[2], F[3], F[4], g1, g2, c,
+                                           1.f / T, (Q11 - Q22) / T, 2.f * Q12 / T);
         const float P11 = P.P11, P12 = P.P12, P21 = P.P21, P22 = P.P22;
         const float det = P11 * P22 - P12 * P21;
         if (!(fabsf(det) > 0.f) || !isfinite(det)) return -1.f;
@@ -923,18 +927,20 @@ __device__ int moment_iterate(const float* s, int h, int w, int npix, const Grp<
     const float inv_tol_pos = 1.f / o.tol_pos, inv_tol_g = 1.f / o.tol_g, inv_tol_sig = 1.f / o.tol_sig;
     int it;
     float m[11];
+    // c = 1 / (2 s_w^2) and the exponent's factor, again only after s_w moved
+    float c = 1.f / (2.f * st.sw * st.sw), cw = -kLog2e / (2.f * st.sw * st.sw);
     // the fourth moments are summed while the ellipticity (or the matched
     // weight size) still moves by more than 1e-3; later passes reuse them
     bool fourth = true;
     for (it = 1; it <= o.max_iter_mom; ++it) {
         const Box bx = weight_box(st, h, w);
         if (fourth)
-            moment_pass<NW, true>(s, w, bx, g, st, m);
+            moment_pass<NW, true>(s, w, bx, g, st, cw, m);
         else
-            moment_pass<NW, false>(s, w, bx, g, st, m);
+            moment_pass<NW, false>(s, w, bx, g, st, cw, m);
 #pragma unroll
         for (int i = 0; i < 5; ++i) F4[i] = m[6 + i];
-        const MomStep d = moment_step(m, st, k_use, ellip, o.sigw_mode == 0);
+        const MomStep d = moment_step(m, st, c, k_use, ellip, o.sigw_mode == 0);
         if (k_use <= 0.f) {
             const float dc = fmaxf(fabsf(d.dx), fabsf(d.dy));
             if (it > 2 && dc >= prev_c) k_use = 0.75f;
@@ -958,13 +964,16 @@ __device__ int moment_iterate(const float* s, int h, int w, int npix, const Grp<
         }
         if (ellip) {
             // |g| < 1: a step past (1 + |g_w|)/2 is shortened radially to it
-            const float cap = 0.5f * (1.f + sqrtf(st.g1 * st.g1 + st.g2 * st.g2));
+            // (at least 1/2, so that a smaller result needs no square root)
             float n1 = st.g1 + d.dg1, n2 = st.g2 + d.dg2;
             const float nn2 = n1 * n1 + n2 * n2;
-            if (nn2 > cap * cap) {
-                const float f = cap * rsqrtf(nn2);
-                n1 *= f;
-                n2 *= f;
+            if (nn2 > 0.25f) {
+                const float cap = 0.5f * (1.f + sqrtf(st.g1 * st.g1 + st.g2 * st.g2));
+                if (nn2 > cap * cap) {
+                    const float f = cap * rsqrtf(nn2);
+                    n1 *= f;
+                    n2 *= f;
+                }
             }
             st.g1 = n1;
             st.g2 = n2;
@@ -978,6 +987,8 @@ __device__ int moment_iterate(const float* s, int h, int w, int npix, const Grp<
             if (ns > sw_max) { ns = sw_max; status |= FSE_ST_SIGW_CLAMPED; }
             dsig = __fdividef(fabsf(ns - st.sw), st.sw);
             st.sw = ns;
+            c = 1.f / (2.f * ns * ns);
+            cw = -kLog2e / (2.f * ns * ns);
         }
         const float xc = static_cast<float>(st.xi) + st.xf, yc = static_cast<float>(st.yi) + st.yf;
         if (st.g1 * st.g1 + st.g2 * st.g2 >= 0.95f * 0.95f || xc < -0.5f ||
@@ -1690,7 +1701,7 @@ __device__ Precise fit_refine(const float* __restrict__ s, const float* __restri
                 for (int ia = 0; ia < sg.S; ++ia) {
                     const float as = sub_a(sg, t1, t2, ia, ic, c0);
                     const float us = exp2_acc(as * inv_n);
-                    const float es = exp2_acc(us * nbl);
+                    const float es = exp2_acc<true>(us * nbl);
                     const float eu = es * us, eua = eu * as, euu = eu * us;
                     E += es;
                     v += eu;
@@ -1753,7 +1764,7 @@ __device__ Precise fit_refine(const float* __restrict__ s, const float* __restri
     for (int p = g.t; p < npix; p += Grp<NW>::NT) {
         const float a = L[p] - c0;
         const float u = exp2_acc(a * inv_n);
-        float E = exp2_acc(u * nbl);
+        float E = exp2_acc<true>(u * nbl);
         float r = fmaf(I0g, E, -s[p]);
         float rr_hi = 0.f, rr_lo = 0.f;
         bool bright = false;
@@ -2190,11 +2201,15 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) es
             st.sw = res.sigma_w;
         } else if (!skip) {
             // centre (and for the fit, ellipticity) from the previous stage
-            bool fin = true;
-            for (int p = g.t; p < npix; p += Grp<NW>::NT) fin = fin && isfinite(s[p]);
-            if (!g.all(fin)) {
-                status |= FSE_ST_NONFINITE;
-                skip = true;
+            // (the chain's start-up has already refused non-finite stamps)
+            if (!(STAGE == kStageFit && a.chain_fit)) {
+                bool fin = true;
+#pragma unroll 4
+                for (int p = g.t; p < npix; p += Grp<NW>::NT) fin = fin && isfinite(s[p]);
+                if (!g.all(fin)) {
+                    status |= FSE_ST_NONFINITE;
+                    skip = true;
+                }
             }
             const float rx = rintf(res.x0), ry = rintf(res.y0);
             st.xi = static_cast<int>(rx);
