@@ -52,6 +52,8 @@ struct LaunchArgs {
     int warps_per_stamp;     // 1, 2, 4 or 8 warps share a stamp (whole chain only)
     int num_ctas;            // 0 = library choice
     int static_assign;       // 1: warp w of the grid takes stamp w only (no counter)
+    int tm_cols;             // fit launches: tensor-memory columns of a warp (set at launch)
+    int tm_alloc;            // ... and of the CTA: a power of two, at least 32 (set at launch)
     int chain_fit;           // kStageFit as the second launch of the chain: keeps every
                              // status bit of the record and fits only converged moments
     // Size-class launches of the ragged path: the launch takes the stamps

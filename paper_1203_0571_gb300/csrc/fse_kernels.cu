@@ -104,6 +104,109 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// ------------------------------------------------------------------ tensor memory
+// The fit keeps one fp32 value per pixel (0.5 log2 R^2) in tensor memory, 256
+// KB per SM that nothing else here uses: lane l of a warp stores the value of
+// its i-th pixel in its own lane, column i, so a store or load of K columns
+// moves K registers per lane (.32x32b.xK).  Warp w of a CTA reaches the 32
+// lanes of quadrant w % 4 only.  The loads are asynchronous: their registers
+// are ready after the wait, which takes them as operands so that no use moves
+// above it.
+__device__ __forceinline__ void tm_store8(uint32_t addr, const float (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr),
+                 "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+__device__ __forceinline__ void tm_wait_store() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[1]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
+                 : "=f"(v[0])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tm_wait(float (&v)[1]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]) : : "memory");
+}
+
+__device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[2]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
+                 : "=f"(v[0]), "=f"(v[1])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tm_wait(float (&v)[2]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]) : : "memory");
+}
+
+__device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tm_wait(float (&v)[4]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]) : : "memory");
+}
+
+__device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tm_wait(float (&v)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
+                 :
+                 : "memory");
+}
+
+// Calls body(p, a) for the thread's pixels p = t, t + NT, ... in order, with
+// a = L - c0 and L the pixel's value from tensor memory.  K columns are loaded
+// at a time, the next ones while the body works on the last; the loaded
+// registers are read after the wait of the same iteration only.  Every warp
+// makes the same loads (they are warp-wide); pixels past the end are skipped.
+template <int K, int NT, typename F>
+__device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0, F body) {
+    const int full = npix / NT;   // columns that hold a pixel of every thread
+    float v[K], a[K];
+    int c = 0;
+    if (full >= K) {
+        __syncwarp();
+        tm_load(tm, v);
+        tm_wait(v);
+#pragma unroll
+        for (int j = 0; j < K; ++j) a[j] = v[j] - c0;
+#pragma unroll 1
+        for (; c + K <= full; c += K) {
+            const int next = c + 2 * K <= full ? c + K : c;   // (the last load is not used)
+            __syncwarp();
+            tm_load(tm + next, v);
+#pragma unroll
+            for (int j = 0; j < K; ++j) body(t + NT * (c + j), a[j]);
+            tm_wait(v);
+#pragma unroll
+            for (int j = 0; j < K; ++j) a[j] = v[j] - c0;
+        }
+    }
+#pragma unroll 1
+    for (; c * NT < npix; ++c) {
+        float u[1];
+        __syncwarp();
+        tm_load(tm + c, u);
+        tm_wait(u);
+        if (t + NT * c < npix) body(t + NT * c, u[0] - c0);
+    }
+}
+
 // ------------------------------------------------------------------ stamp groups
 // NW warps may share one stamp (large stamps, whose shared-memory tile leaves
 // room for few of them per SM).  Thread t = 32 (warp in group) + lane strides
@@ -309,19 +412,15 @@ __global__ void eval_bn_kernel(const double* n, double* b, double* db, int64_t c
 }
 
 // ------------------------------------------------------------------ per-warp layout
-// [pixels: max_pix + 4 floats][aux: max(max_pix, 512) floats][ivar: max_pix + 4 (opt)][mbarrier]
+// [pixels: max_pix + 4 floats][aux][ivar: max_pix + 4 (opt)][mbarrier]
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 __host__ __device__ inline size_t pix_bytes(int max_pix) { return align16((size_t)(max_pix + 4) * 4); }
-__host__ __device__ inline size_t aux_bytes(int max_pix) {
-    return align16((size_t)(max_pix > 512 ? max_pix : 512) * 4);
-}
-__host__ __device__ inline size_t warp_bytes(int max_pix, bool ivar) {
-    return pix_bytes(max_pix) + aux_bytes(max_pix) + (ivar ? pix_bytes(max_pix) : 0) + 16;
-}
-// Shared memory of a stamp group: the tile above plus, for nw > 1 warps per
-// stamp, the reduction scratch (nw x 32 words) and the work-counter word.
-__host__ __device__ inline size_t group_bytes(int max_pix, bool ivar, int nw) {
-    return warp_bytes(max_pix, ivar) + (nw > 1 ? static_cast<size_t>(nw) * 128 + 16 : 0);
+// The tile size by which launch shapes are chosen, accepted and saved
+// (smem_per_group): pixels, one more float per pixel, inverse variance.  No
+// stage takes more.
+__host__ __device__ inline size_t shape_bytes(int max_pix, bool ivar, int nw) {
+    return pix_bytes(max_pix) + align16((size_t)(max_pix > 512 ? max_pix : 512) * 4) +
+           (ivar ? pix_bytes(max_pix) : 0) + 16 + (nw > 1 ? static_cast<size_t>(nw) * 128 + 16 : 0);
 }
 
 // Rings the start-up's growth curve can need for stamps of at most max_pix
@@ -343,28 +442,26 @@ inline int ring_slots(int max_pix) {
     return k + 2;
 }
 
-// The moment stages keep a smaller tile: the pixels, and an auxiliary area
-// only for the raw bf16 staging and, in the start-up launch, the ring
-// histogram (three 32-bit words per ring); no inverse variance (the moments do
-// not use it).  For 48x48 fp32 that is 9.2 KB per warp in the moment launch
-// and 10.8 KB in the start-up, instead of the fit's 18.5 KB.
-__host__ __device__ inline size_t aux_bytes_moments(int max_pix, bool bf16, int slots) {
-    const size_t raw = bf16 ? static_cast<size_t>(max_pix + 8) * 2 : 0;
-    const size_t hist = static_cast<size_t>(slots) * 12;
-    return align16(raw > hist ? raw : hist);
-}
+// What a launch takes per warp: the pixels, an auxiliary area only for the raw
+// bf16 staging and, in the start-up launch, the ring histogram (three 32-bit
+// words per ring), and the inverse variance in the fit (the moments do not use
+// it).  For 48x48 fp32 that is 9.2 KB per warp in the moment and fit launches
+// and 10.8 KB in the start-up.
 __host__ __device__ inline constexpr bool moment_stage(int stage) {
     return stage == kStageCentroid || stage == kStageEllipticity || stage == kStageMoments ||
            stage == kStageStartup;
 }
 __host__ __device__ inline size_t stage_aux_bytes(int stage, int max_pix, bool bf16, int slots) {
-    return moment_stage(stage) ? aux_bytes_moments(max_pix, bf16, stage == kStageStartup ? slots : 0)
-                               : aux_bytes(max_pix);
+    const size_t raw = bf16 ? static_cast<size_t>(max_pix + 8) * 2 : 0;
+    const size_t hist = stage == kStageStartup ? static_cast<size_t>(slots) * 12 : 0;
+    return align16(raw > hist ? raw : hist);
 }
 __host__ __device__ inline size_t stage_warp_bytes(int stage, int max_pix, bool bf16, bool ivar, int slots) {
     return pix_bytes(max_pix) + stage_aux_bytes(stage, max_pix, bf16, slots) +
            (ivar && !moment_stage(stage) ? pix_bytes(max_pix) : 0) + 16;
 }
+// Shared memory of a stamp group: the tile above plus, for nw > 1 warps per
+// stamp, the reduction scratch (nw x 32 words) and the work-counter word.
 __host__ __device__ inline size_t stage_group_bytes(int stage, int max_pix, bool bf16, bool ivar, int nw,
                                                     int slots) {
     return stage_warp_bytes(stage, max_pix, bf16, ivar, slots) +
@@ -1371,7 +1468,7 @@ struct FitEval {
 };
 
 template <bool IVAR, int NW, bool SUP = false>
-__device__ FitEval fit_eval(const float* __restrict__ s, const float* __restrict__ L,
+__device__ FitEval fit_eval(const float* __restrict__ s, uint32_t tm,
                             const float* __restrict__ sq, int npix, const Grp<NW>& g, float I0g,
                             float re, float n, float lq, int w = 0, const MomState* st = nullptr,
                             int S = 1) {
@@ -1383,19 +1480,27 @@ __device__ FitEval fit_eval(const float* __restrict__ s, const float* __restrict
     float acc[10];
 #pragma unroll
     for (int i = 0; i < 10; ++i) acc[i] = 0.f;
-    SubGeom sg;
-    if constexpr (SUP) sg = sub_geom(*st, S);
-    PixelWalk pw(g.t, SUP ? w : 1, Grp<NW>::NT);
-    // four pixels in flight: their exp2 chains overlap, which the fit launch's
-    // 12 warps per SM do not hide alone (2% faster than two)
-#pragma unroll 4
-    for (int p = g.t; p < npix; p += Grp<NW>::NT) {
-        float E, v = 0.f, va = 0.f, u = 0.f, a = 0.f;
-        if constexpr (SUP) {
+    // the ten sums of one pixel; E, r and (v, va) already carry sqrt(inv_var)
+    auto add = [&](float E, float r, float v, float va) {
+        acc[0] = fmaf(E, E, acc[0]);
+        acc[1] = fmaf(E, v, acc[1]);
+        acc[2] = fmaf(E, va, acc[2]);
+        acc[3] = fmaf(v, v, acc[3]);
+        acc[4] = fmaf(v, va, acc[4]);
+        acc[5] = fmaf(va, va, acc[5]);
+        acc[6] = fmaf(E, r, acc[6]);
+        acc[7] = fmaf(v, r, acc[7]);
+        acc[8] = fmaf(va, r, acc[8]);
+        acc[9] = fmaf(r, r, acc[9]);
+    };
+    if constexpr (SUP) {
+        const SubGeom sg = sub_geom(*st, S);
+        PixelWalk pw(g.t, w, Grp<NW>::NT);
+        for (int p = g.t; p < npix; p += Grp<NW>::NT) {
+            float E = 0.f, v = 0.f, va = 0.f;
             float t1, t2;
             pix_t(pw, *st, &t1, &t2);
             pw.next();
-            E = 0.f;
             for (int ic = 0; ic < sg.S; ++ic)
                 for (int ia = 0; ia < sg.S; ++ia) {
                     const float as = sub_a(sg, t1, t2, ia, ic, c0);
@@ -1408,35 +1513,31 @@ __device__ FitEval fit_eval(const float* __restrict__ s, const float* __restrict
             E *= sg.invS2;
             v *= sg.invS2;
             va *= sg.invS2;
-        } else {
-            a = L[p] - c0;
-            u = ex2(a * inv_n);
-            E = ex2(u * nbl);
-        }
-        float r = fmaf(I0g, E, -s[p]);
-        if (IVAR) {
-            const float q = sq[p];
-            E *= q;
-            r *= q;
-            if constexpr (SUP) {
+            float r = fmaf(I0g, E, -s[p]);
+            if (IVAR) {
+                const float q = sq[p];
+                E *= q;
+                r *= q;
                 v *= q;
                 va *= q;
             }
+            add(E, r, v, va);
         }
-        if constexpr (!SUP) {
-            v = E * u;
-            va = v * a;
-        }
-        acc[0] = fmaf(E, E, acc[0]);
-        acc[1] = fmaf(E, v, acc[1]);
-        acc[2] = fmaf(E, va, acc[2]);
-        acc[3] = fmaf(v, v, acc[3]);
-        acc[4] = fmaf(v, va, acc[4]);
-        acc[5] = fmaf(va, va, acc[5]);
-        acc[6] = fmaf(E, r, acc[6]);
-        acc[7] = fmaf(v, r, acc[7]);
-        acc[8] = fmaf(va, r, acc[8]);
-        acc[9] = fmaf(r, r, acc[9]);
+    } else {
+        // eight pixels at a time: their exp2 chains overlap (four with eight warps
+        // per stamp, whose smaller stamps have only four pixels a thread)
+        tm_pixels<NW >= 8 ? 4 : 8, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) {
+            const float u = ex2(a * inv_n);
+            float E = ex2(u * nbl);
+            float r = fmaf(I0g, E, -s[p]);
+            if (IVAR) {
+                const float q = sq[p];
+                E *= q;
+                r *= q;
+            }
+            const float v = E * u;
+            add(E, r, v, v * a);
+        });
     }
     g.allsum(acc);
     FitEval f;
@@ -1465,7 +1566,7 @@ __device__ FitEval fit_eval(const float* __restrict__ s, const float* __restrict
 // Start: r_e from the weight size, n the candidate of {0.5, 1, 2, 4} with the
 // lowest chi^2 at its closed-form I0 (chi^2 = sum I^2 - (sum I E)^2 / sum E^2).
 template <bool IVAR, int NW, bool SUP = false>
-__device__ void fit_start(const float* __restrict__ s, const float* __restrict__ L,
+__device__ void fit_start(const float* __restrict__ s, uint32_t tm,
                           const float* __restrict__ sq, int npix, const Grp<NW>& g, float re0,
                           float lq, float* n0, float* I00, int w = 0, const MomState* st = nullptr,
                           int S = 1) {
@@ -1482,15 +1583,14 @@ __device__ void fit_start(const float* __restrict__ s, const float* __restrict__
     float acc[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) acc[i] = 0.f;
-    SubGeom sg;
-    if constexpr (SUP) sg = sub_geom(*st, S);
-    PixelWalk pw(g.t, SUP ? w : 1, Grp<NW>::NT);
-    for (int p = g.t; p < npix; p += Grp<NW>::NT) {
-        float I = s[p];
-        const float q = IVAR ? sq[p] : 1.f;
-        if (IVAR) I *= q;
-        acc[8] = fmaf(I, I, acc[8]);
-        if constexpr (SUP) {
+    if constexpr (SUP) {
+        const SubGeom sg = sub_geom(*st, S);
+        PixelWalk pw(g.t, w, Grp<NW>::NT);
+        for (int p = g.t; p < npix; p += Grp<NW>::NT) {
+            float I = s[p];
+            const float q = IVAR ? sq[p] : 1.f;
+            if (IVAR) I *= q;
+            acc[8] = fmaf(I, I, acc[8]);
             float t1, t2;
             pix_t(pw, *st, &t1, &t2);
             pw.next();
@@ -1508,8 +1608,13 @@ __device__ void fit_start(const float* __restrict__ s, const float* __restrict__
                 acc[2 * c] = fmaf(E, E, acc[2 * c]);
                 acc[2 * c + 1] = fmaf(E, I, acc[2 * c + 1]);
             }
-        } else {
-            const float a = L[p] - c0;
+        }
+    } else {
+        tm_pixels<2, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) {
+            float I = s[p];
+            const float q = IVAR ? sq[p] : 1.f;
+            if (IVAR) I *= q;
+            acc[8] = fmaf(I, I, acc[8]);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 float E = ex2(ex2(a * inv_n[c]) * nbl[c]);
@@ -1517,7 +1622,7 @@ __device__ void fit_start(const float* __restrict__ s, const float* __restrict__
                 acc[2 * c] = fmaf(E, E, acc[2 * c]);
                 acc[2 * c + 1] = fmaf(E, I, acc[2 * c + 1]);
             }
-        }
+        });
     }
     g.allsum(acc);
     int best = 0;
@@ -1659,7 +1764,7 @@ __device__ Precise refine_tail(const float (&rh)[10], const float (&rl)[10], con
 }
 
 template <bool IVAR, int NW, bool SUP = false>
-__device__ Precise fit_refine(const float* __restrict__ s, const float* __restrict__ L,
+__device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
                               const float* __restrict__ sq, int w, int npix, const Grp<NW>& g,
                               float I0g,
                               float re, float n, float lq, const MomState& st, int S = 1) {
@@ -1760,55 +1865,55 @@ __device__ Precise fit_refine(const float* __restrict__ s, const float* __restri
                 df_add(rh[9], rl[9], r * r);
             }
         }
-    } else
-    for (int p = g.t; p < npix; p += Grp<NW>::NT) {
-        const float a = L[p] - c0;
-        const float u = exp2_acc(a * inv_n);
-        float E = exp2_acc<true>(u * nbl);
-        float r = fmaf(I0g, E, -s[p]);
-        float rr_hi = 0.f, rr_lo = 0.f;
-        bool bright = false;
-        if (check_bright) {
-            const float q = IVAR ? sq[p] : 1.f;
-            if (fabsf(I0g * E) * q > kBrightSigma) {
-                const double rrd = bright_r2(bm, static_cast<double>(pw.col - st.xi) - st.xf,
-                                             static_cast<double>(pw.row - st.yi) - st.yf, s[p], q);
-                rr_hi = static_cast<float>(rrd);
-                rr_lo = static_cast<float>(rrd - rr_hi);
-                bright = true;
+    } else {
+        tm_pixels<1, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) {
+            const float u = exp2_acc(a * inv_n);
+            float E = exp2_acc<true>(u * nbl);
+            float r = fmaf(I0g, E, -s[p]);
+            float rr_hi = 0.f, rr_lo = 0.f;
+            bool bright = false;
+            if (check_bright) {
+                const float q = IVAR ? sq[p] : 1.f;
+                if (fabsf(I0g * E) * q > kBrightSigma) {
+                    const double rrd = bright_r2(bm, static_cast<double>(pw.col - st.xi) - st.xf,
+                                                 static_cast<double>(pw.row - st.yi) - st.yf, s[p], q);
+                    rr_hi = static_cast<float>(rrd);
+                    rr_lo = static_cast<float>(rrd - rr_hi);
+                    bright = true;
+                }
+                pw.next();
             }
-            pw.next();
-        }
-        if (IVAR) {
-            const float q = sq[p];
-            E *= q;
-            r *= q;
-        }
-        const float v = E * u, va = v * a;
-        const float vr = v * r, var = va * r;
-        // J^T J (the first six sums) only shapes the Newton step: fp32.  The
-        // gradient sums and chi^2, which cancel or must hold 1e-7 at the
-        // optimum, are double-float.
-        rh[0] = fmaf(E, E, rh[0]);
-        rh[1] = fmaf(E, v, rh[1]);
-        rh[2] = fmaf(E, va, rh[2]);
-        rh[3] = fmaf(v, v, rh[3]);
-        rh[4] = fmaf(v, va, rh[4]);
-        rh[5] = fmaf(va, va, rh[5]);
-        df_add(rh[6], rl[6], E * r);
-        df_add(rh[7], rl[7], vr);
-        df_add(rh[8], rl[8], var);
-        // residual-weighted second-derivative sums of the model (Newton term)
-        T[0] = fmaf(var, a, T[0]);       // r E u a^2
-        T[1] = fmaf(vr, u, T[1]);        // r E u^2
-        T[2] = fmaf(var, u, T[2]);       // r E u^2 a
-        T[3] = fmaf(var * u, a, T[3]);   // r E u^2 a^2
-        if (bright) {
-            df_add(rh[9], rl[9], rr_hi);
-            rl[9] += rr_lo;
-        } else {
-            df_add(rh[9], rl[9], r * r);
-        }
+            if (IVAR) {
+                const float q = sq[p];
+                E *= q;
+                r *= q;
+            }
+            const float v = E * u, va = v * a;
+            const float vr = v * r, var = va * r;
+            // J^T J (the first six sums) only shapes the Newton step: fp32.  The
+            // gradient sums and chi^2, which cancel or must hold 1e-7 at the
+            // optimum, are double-float.
+            rh[0] = fmaf(E, E, rh[0]);
+            rh[1] = fmaf(E, v, rh[1]);
+            rh[2] = fmaf(E, va, rh[2]);
+            rh[3] = fmaf(v, v, rh[3]);
+            rh[4] = fmaf(v, va, rh[4]);
+            rh[5] = fmaf(va, va, rh[5]);
+            df_add(rh[6], rl[6], E * r);
+            df_add(rh[7], rl[7], vr);
+            df_add(rh[8], rl[8], var);
+            // residual-weighted second-derivative sums of the model (Newton term)
+            T[0] = fmaf(var, a, T[0]);       // r E u a^2
+            T[1] = fmaf(vr, u, T[1]);        // r E u^2
+            T[2] = fmaf(var, u, T[2]);       // r E u^2 a
+            T[3] = fmaf(var * u, a, T[3]);   // r E u^2 a^2
+            if (bright) {
+                df_add(rh[9], rl[9], rr_hi);
+                rl[9] += rr_lo;
+            } else {
+                df_add(rh[9], rl[9], r * r);
+            }
+        });
     }
     g.allsum_df(rh, rl);
     g.allsum(T);
@@ -1833,7 +1938,7 @@ struct FitOut {
 // Levenberg-Marquardt over theta = (r_e, n) with I0 at its closed form after
 // every pass; damping by the gain ratio rho (Nielsen 1999).
 template <bool IVAR, int NW, bool SUP = false>
-__device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, int w, int npix,
+__device__ FitOut sersic_fit(const float* s, uint32_t tm, const float* sq, int h, int w, int npix,
                              const Grp<NW>& g, const DevOpts& o, const MomState& st,
                              uint32_t& status) {
     // per-pixel 0.5 log2 R^2 about the fixed centre with the fixed ellipticity
@@ -1843,15 +1948,23 @@ __device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, i
     const float A = 1.f + gg - 2.f * g1, B = 1.f + gg + 2.f * g1, G4 = 4.f * g2;
     const int S = SUP ? o.supersample : 1;
     if constexpr (!SUP) {
+        // eight columns of tensor memory at a time (the last ones may lie past
+        // the stamp: values of no pixel, never read back)
         PixelWalk pw(g.t, w, Grp<NW>::NT);
-        for (int p = g.t; p < npix; p += Grp<NW>::NT) {
-            const float t1 = static_cast<float>(pw.col - st.xi) - st.xf;
-            const float t2 = static_cast<float>(pw.row - st.yi) - st.yf;
-            const float R2 = fmaf(A, t1 * t1, fmaf(B, t2 * t2, -G4 * (t1 * t2)));
-            L[p] = half_log2_r2(R2);
-            pw.next();
+#pragma unroll 1
+        for (int c = 0; c * Grp<NW>::NT < npix; c += 8) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float t1 = static_cast<float>(pw.col - st.xi) - st.xf;
+                const float t2 = static_cast<float>(pw.row - st.yi) - st.yf;
+                const float R2 = fmaf(A, t1 * t1, fmaf(B, t2 * t2, -G4 * (t1 * t2)));
+                v[j] = half_log2_r2(R2);
+                pw.next();
+            }
+            tm_store8(tm + c, v);
         }
-        g.sync();
+        tm_wait_store();
     }
     const float gabs = sqrtf(gg);
     const float lq = log2f(1.f - gabs);          // log2 r = 0.5 log2 R^2 - log2(1 - |g|)
@@ -1860,7 +1973,7 @@ __device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, i
     float re = static_cast<float>(kSqrt2Ln2) * st.sw / (1.f - gabs);
     re = re < re_min ? re_min : (re > re_max ? re_max : re);
     float n, I0g;
-    fit_start<IVAR, NW, SUP>(s, L, sq, npix, g, re, lq, &n, &I0g, w, &st, S);
+    fit_start<IVAR, NW, SUP>(s, tm, sq, npix, g, re, lq, &n, &I0g, w, &st, S);
     // One evaluation site: every pass of the profile goes through the single
     // fit_eval call at the top of this loop (first the start, then each trial
     // step, and a repeat at I0* when the amplitude jumped).
@@ -1872,7 +1985,7 @@ __device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, i
     int evals = 0, band_accepts = 0, it = 0;
 #pragma unroll 1
     for (;;) {
-        const FitEval ev = fit_eval<IVAR, NW, SUP>(s, L, sq, npix, g, I0t, ret, nt, lq, w, &st, S);
+        const FitEval ev = fit_eval<IVAR, NW, SUP>(s, tm, sq, npix, g, I0t, ret, nt, lq, w, &st, S);
         ++evals;
         if (ev.corr > 0.5f && !retried) {
             // the amplitude moved so far that chi^2 lost precision: evaluate again at I0*
@@ -1970,7 +2083,7 @@ __device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, i
         int passes = 0;
 #pragma unroll 1
         for (;;) {
-            const Precise E = fit_refine<IVAR, NW, SUP>(s, L, sq, w, npix, g, tI0, te, tn, lq, st, S);
+            const Precise E = fit_refine<IVAR, NW, SUP>(s, tm, sq, w, npix, g, tI0, te, tn, lq, st, S);
             ++passes;
             // a step within 1e-2 is taken on the Newton model alone: its chi^2
             // decrease can be below the rounding of the fp32 model values
@@ -2032,14 +2145,16 @@ __device__ FitOut sersic_fit(const float* s, float* L, const float* sq, int h, i
 // NW warps share each stamp (a stamp group); a CTA holds blockDim.x / (32 NW)
 // groups, each with its own tile and, for NW > 1, named barrier 1 + group.
 template <int STAGE, int DT, bool IVAR, int NW, bool SUP = false>
-// Fit stages: 168 registers per thread let three CTAs of four warps share an
-// SM (the launch shape of 48x48 and smaller tiles); more would leave two.
+// Fit stages: 128 registers per thread let four CTAs of four warps share an SM
+// (two of eight warps), which tensor memory (128 of 512 columns each for 48x48)
+// and the 9.2 KB tiles allow too.  The pixel-integrated model, whose sub-grid
+// loops spill at 168, keeps those.
 // Moment stages and the start-up: 96 registers (they spill nothing at 96) let
 // five CTAs of four warps share an SM with their compact tile.  With eight
 // warps per stamp (the 128x128 tiles) the tile already limits an SM to two
 // CTAs of 256 threads, so 128 registers cost no occupancy and keep the group
 // reductions of the refinement pass out of local memory.
-__global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) estimator_kernel(LaunchArgs a) {
+__global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 168 : 128)) estimator_kernel(LaunchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -2070,6 +2185,23 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) es
     g.sync();
     uint32_t phase = 0;
     const DevOpts& o = a.opts;
+    // the fit's tensor memory: one allocation per CTA, released at the end by
+    // the same warp; a warp's columns start at tm in its quadrant's lanes
+    constexpr bool kTm = STAGE == kStageFit && !SUP;
+    __shared__ uint32_t tm_base;
+    uint32_t tm = 0;
+    if constexpr (kTm) {
+        if (warp == 0) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tm_base)),
+                         "r"(a.tm_alloc)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tm = tm_base + (static_cast<uint32_t>(warp & 3) << 21) + static_cast<uint32_t>((warp >> 2) * a.tm_cols);
+    }
     // this launch's stamps: all of them, or one size class through perm
     const unsigned long long count = a.range ? a.range[1] : static_cast<unsigned long long>(a.count);
     const unsigned base = a.range ? a.range[0] : 0u;
@@ -2161,7 +2293,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) es
                     res.status = status | FSE_ST_TIMEOUT;
                     a.out[si] = res;
                 }
-                return;
+                break;
             }
         }
         const int npix = static_cast<int>(npl);
@@ -2250,7 +2382,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) es
             }
         }
         if (!skip && (STAGE == kStageFit || STAGE == kStageAll)) {
-            const FitOut f = sersic_fit<IVAR, NW, SUP>(s, aux, ivbuf, h, w, npix, g, o, st, status);
+            const FitOut f = sersic_fit<IVAR, NW, SUP>(s, tm, ivbuf, h, w, npix, g, o, st, status);
             res.I0 = static_cast<float>(f.I0);
             res.re = static_cast<float>(f.re);
             res.n = static_cast<float>(f.n);
@@ -2262,16 +2394,40 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : 168) es
         if (g.t == 0) a.out[si] = res;
         g.sync();
     }
+    if constexpr (kTm) {
+        // every warp's loads and stores are done (each waited for its own)
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (warp == 0)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm_base), "r"(a.tm_alloc)
+                         : "memory");
+    }
 }
 
 template <int STAGE, int DT, bool IVAR, int NW, bool SUP = false>
 cudaError_t launch_t(const LaunchArgs& a_in, cudaStream_t stream) {
     LaunchArgs a = a_in;
     a.opts.ring_slots = ring_slots(a.opts.max_pix);
-    const int groups = a.warps_per_cta / NW;
+    int groups = a.warps_per_cta / NW;
     if (groups < 1 || groups * NW != a.warps_per_cta || groups > 15) return cudaErrorInvalidValue;
-    const size_t smem =
-        stage_group_bytes(STAGE, a.opts.max_pix, DT == FSE_BF16, IVAR, NW, a.opts.ring_slots) * groups;
+    const size_t spg = stage_group_bytes(STAGE, a.opts.max_pix, DT == FSE_BF16, IVAR, NW, a.opts.ring_slots);
+    if constexpr (STAGE == kStageFit && !SUP) {
+        // Tensor memory is allocated in columns over all four quadrants, so a
+        // CTA of fewer than four warps would leave the other quadrants' lanes
+        // idle: such a shape is widened to four warps as far as shared memory
+        // allows (groups are independent; the results do not depend on it).
+        if (shape_bytes(a.opts.max_pix, IVAR, NW) * groups > 227 * 1024) return cudaErrorInvalidValue;
+        if (!a.static_assign)
+            while (groups * NW < 4 && spg * (2 * groups) <= 226 * 1024) groups *= 2;
+        a.warps_per_cta = groups * NW;
+        a.tm_cols = (((a.opts.max_pix + 32 * NW - 1) / (32 * NW)) + 7) & ~7;
+        const int cols = a.tm_cols * ((a.warps_per_cta + 3) / 4);
+        a.tm_alloc = 32;
+        while (a.tm_alloc < cols) a.tm_alloc *= 2;
+        if (a.tm_alloc > 512) return cudaErrorInvalidConfiguration;
+    }
+    const size_t smem = spg * groups;
     auto kern = estimator_kernel<STAGE, DT, IVAR, NW, SUP>;
     // the shared-memory opt-in is raised once per instantiation and size (per
     // device and context: a device reset clears it)
@@ -2298,6 +2454,17 @@ cudaError_t launch_t(const LaunchArgs& a_in, cudaStream_t stream) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * a.warps_per_cta, smem);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        if (STAGE == kStageFit && !SUP) {
+            // the occupancy calculator answers one CTA per SM for any kernel
+            // that allocates tensor memory; the limits are registers (128 a
+            // thread), shared memory (228 KB with 1 KB per CTA) and columns
+            const int by_regs = 512 / (32 * a.warps_per_cta);
+            const int by_smem = static_cast<int>(228 * 1024 / (smem + 1024 + 16));
+            per_sm = 512 / a.tm_alloc;
+            per_sm = by_regs < per_sm ? by_regs : per_sm;
+            per_sm = by_smem < per_sm ? by_smem : per_sm;
+            if (per_sm < 1) per_sm = 1;
+        }
         grid = static_cast<long long>(per_sm) * sms;
     }
     const long long need = (a.count + groups - 1) / groups;
@@ -2379,14 +2546,14 @@ unsigned long long current_context_id() {
 }
 
 size_t smem_per_group(int max_pix, bool ivar, int warps_per_stamp) {
-    return group_bytes(max_pix, ivar, warps_per_stamp);
+    return shape_bytes(max_pix, ivar, warps_per_stamp);
 }
 
 void choose_launch(int max_pix, int* warps_per_cta, int* warps_per_stamp) {
     // one warp per stamp up to 48x48 tiles; larger tiles leave room for few
     // stamps per SM, so several warps share each of them
     const int nw = max_pix <= 48 * 48 ? 1 : max_pix <= 64 * 64 ? 2 : max_pix <= 96 * 96 ? 4 : 8;
-    const size_t spg = group_bytes(max_pix, false, nw);
+    const size_t spg = shape_bytes(max_pix, false, nw);
     const size_t budget = 227 * 1024;
     int groups = nw == 1 ? 4 : 1;
     while (groups > 1 && spg * groups > budget) groups >>= 1;
