@@ -171,15 +171,16 @@ __device__ __forceinline__ void tm_wait(float (&v)[8]) {
 
 // Calls body(p, a) for the thread's pixels p = t, t + NT, ... in order, with
 // a = L - c0 and L the pixel's value from tensor memory.  K columns are loaded
-// at a time, the next ones while the body works on the last; the loaded
-// registers are read after the wait of the same iteration only.  Every warp
-// makes the same loads (they are warp-wide); pixels past the end are skipped.
+// at a time, the next ones while the body works on the last (the loaded
+// registers are read after the wait of the same iteration only); then the
+// columns left over, two at a time and one at a time.  Every warp makes the
+// same loads (they are warp-wide); pixels past the end are skipped.
 template <int K, int NT, typename F>
 __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0, F body) {
     const int full = npix / NT;   // columns that hold a pixel of every thread
-    float v[K], a[K];
     int c = 0;
     if (full >= K) {
+        float v[K], a[K];
         __syncwarp();
         tm_load(tm, v);
         tm_wait(v);
@@ -197,13 +198,24 @@ __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0
             for (int j = 0; j < K; ++j) a[j] = v[j] - c0;
         }
     }
+    if constexpr (K > 2) {
+#pragma unroll 1
+        for (; c + 2 <= full; c += 2) {
+            float v[2];
+            __syncwarp();
+            tm_load(tm + c, v);
+            tm_wait(v);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) body(t + NT * (c + j), v[j] - c0);
+        }
+    }
 #pragma unroll 1
     for (; c * NT < npix; ++c) {
-        float u[1];
+        float v[1];
         __syncwarp();
-        tm_load(tm + c, u);
-        tm_wait(u);
-        if (t + NT * c < npix) body(t + NT * c, u[0] - c0);
+        tm_load(tm + c, v);
+        tm_wait(v);
+        if (t + NT * c < npix) body(t + NT * c, v[0] - c0);
     }
 }
 
