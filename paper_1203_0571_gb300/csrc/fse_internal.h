@@ -188,7 +188,7 @@ cudaError_t eval_bn(const double* n, double* b, double* db, int64_t count, cudaS
 cudaError_t launch_estimator(const LaunchArgs& a, cudaStream_t stream);
 // Launches the implicit-gradient kernel; returns the launch error.
 cudaError_t launch_moment_grad(const MomentGradArgs& a, cudaStream_t stream);
-// Launches the three cut-out kernels; returns the launch error.
+// Launches the cut-out kernels; returns the launch error.
 cudaError_t launch_cutout(const CutoutArgs& a, cudaStream_t stream);
 // Launches the star-profile kernel; returns the launch error.
 cudaError_t launch_star(const StarArgs& a, cudaStream_t stream);

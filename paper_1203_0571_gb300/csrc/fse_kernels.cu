@@ -1154,86 +1154,6 @@ struct InitOut {
     bool overflow;   // the stamp needs more rings than the tile holds (not expected)
 };
 
-// ceil(sqrt(d2)) for an integer 0 <= d2 <= 2 * 127^2 (sides of at most
-// FSE_MAX_SIDE = 128 pixels), with one MUFU operation and integer arithmetic:
-// d2 becomes a float through the bits of 2^23 + d2 (exact below 2^23), and the
-// root is rounded to the nearest integer k0 by adding 2^23 (whose ulp is 1).
-// sqrt.approx.f32 is within about 2^-22 relative of the square root, under
-// 1e-4 here, so k0 is the floor or the ceiling of the true root, and the
-// comparison k0^2 < d2 turns either into the ceiling.
-__device__ __forceinline__ int ring_of(int d2) {
-    const float f = __int_as_float(0x4B000000 | d2) - 8388608.f;
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(f));
-    const int k0 = __float_as_int(r + 8388608.f) - 0x4B000000;
-    return k0 + (k0 * k0 < d2 ? 1 : 0);
-}
-
-// Fixed-point pieces of a pixel.  The growth curve sums q = rn(v 2^S), a
-// 64-bit integer, exactly.  q = q2 2^(2B) + q1 2^B + q0 with signed pieces
-// |q0|, |q1| <= 2^(B-1): no piece's sum over the stamp can leave 32 bits, so
-// native 32-bit adds (registers, shared-memory atomics) hold them exactly.
-// Each piece is the nearest integer to what is left of v, by adding
-// 1.5 2^23 (exact to nearest even for magnitudes up to 2^22) with the scaling
-// in the same FMA; the remainders are exact, and 2^B is even, so the last
-// rounding is that of the whole value.  Three FMAs and a subtraction per
-// piece replace the 64-bit conversion instruction, which issues once in about
-// 17 cycles of an SM on this chip's fp64 pipe.
-struct FixScale {
-    float up2, up1, up0;   // 2^(S - 2B), 2^(S - B), 2^S
-    float dn2, dn1;        // -2^(2B - S), -2^(B - S)
-    int B;
-    bool wide;             // the scale does not bound q: convert in 64 bits
-};
-
-__device__ __forceinline__ FixScale fix_scale(float amax, int npix) {
-    // amax * npix * 2^S < 2^62
-    int e;
-    const float top = amax * static_cast<float>(npix);
-    frexpf(top, &e);
-    int S = 62 - e;
-    S = S > 100 ? 100 : (S < -100 ? -100 : S);
-    // 31 - ceil(log2 npix) bits a piece, and at most 22 (q0 and q1 from the
-    // rounding adds); then |q2| <= 2^(62 - 2B) / npix is below 2^22 too
-    const int b = 31 - (npix > 1 ? 32 - __clz(npix - 1) : 0);
-    FixScale f;
-    f.B = b < 22 ? b : 22;
-    f.up0 = ldexpf(1.f, S);
-    f.up1 = ldexpf(1.f, S - f.B);
-    f.up2 = ldexpf(1.f, S - 2 * f.B);
-    f.dn2 = -ldexpf(1.f, 2 * f.B - S);
-    f.dn1 = -ldexpf(1.f, f.B - S);
-    f.wide = !(top < INFINITY);
-    return f;
-}
-
-// The pieces plus 0x4B400000 each (the bits of 1.5 2^23 + piece); with `wide`
-// the pieces of the saturated 64-bit conversion in the same form.
-constexpr int kFixBias = 0x4B400000;
-__device__ __forceinline__ void fix_split(const FixScale& f, float v, int& q0, int& q1, int& q2) {
-    constexpr float kRound = 12582912.f;
-    const float z2 = fmaf(v, f.up2, kRound);
-    const float r1 = fmaf(__fsub_rn(z2, kRound), f.dn2, v);
-    const float z1 = fmaf(r1, f.up1, kRound);
-    const float r0 = fmaf(__fsub_rn(z1, kRound), f.dn1, r1);
-    const float z0 = fmaf(r0, f.up0, kRound);
-    q2 = __float_as_int(z2);
-    q1 = __float_as_int(z1);
-    q0 = __float_as_int(z0);
-    if (f.wide) {
-        const long long q = __float2ll_rn(v * f.up0);
-        const long long m = (1ll << f.B) - 1;
-        q0 = static_cast<int>(q & m) + kFixBias;
-        q1 = static_cast<int>((q >> f.B) & m) + kFixBias;
-        q2 = static_cast<int>(q >> (2 * f.B)) + kFixBias;
-    }
-}
-
-__device__ __forceinline__ long long fix_join(const FixScale& f, int s0, int s1, int s2) {
-    return static_cast<long long>(s0) + static_cast<long long>(s1) * (1ll << f.B) +
-           static_cast<long long>(static_cast<unsigned long long>(static_cast<long long>(s2)) << (2 * f.B));
-}
-
 // Brightest pixel, and the half-light radius r50 from the growth curve around
 // it (Sec. 4.1): pixels are binned in rings of integer radius k (k-1 < d <= k)
 // and the enclosed sum is tracked until it reaches half the stamp total; r50
@@ -1293,7 +1213,9 @@ __device__ InitOut stamp_init(const float* s, int h, int w, int npix, const Grp<
     o.r50 = static_cast<float>(kSqrt2Ln2);
     if (!o.finite) return o;
     const int pr = imax / w, pc = imax - (imax / w) * w;
-    const FixScale fx = fix_scale(__uint_as_float(ab), npix);
+    // pieces whose sums over the stamp fit 32 bits: 31 - ceil(log2 npix) bits
+    const int bits = 31 - (npix > 1 ? 32 - __clz(npix - 1) : 0);
+    const FixScale fx = fix_scale(__uint_as_float(ab), npix, bits < 22 ? bits : 22);
     // the largest row and column distance from the brightest pixel to an edge
     const int dh = (h - 1 - pr > pr ? h - 1 - pr : pr), dw = (w - 1 - pc > pc ? w - 1 - pc : pc);
     const int kmax = static_cast<int>(ceilf(sqrtf(static_cast<float>(dh * dh + dw * dw)))) + 1;
@@ -1304,14 +1226,26 @@ __device__ InitOut stamp_init(const float* s, int h, int w, int npix, const Grp<
     long long tot;
     {
         int t0 = 0, t1 = 0, t2 = 0, n = 0;
+        if (!fx.wide) {
 #pragma unroll 4
-        for (int p = g.t; p < npix; p += NT) {
-            int q0, q1, q2;
-            fix_split(fx, s[p], q0, q1, q2);
-            t0 += q0;
-            t1 += q1;
-            t2 += q2;
-            ++n;
+            for (int p = g.t; p < npix; p += NT) {
+                int q0, q1, q2;
+                fix_split3(fx, s[p], q0, q1, q2);
+                t0 += q0;
+                t1 += q1;
+                t2 += q2;
+                ++n;
+            }
+        } else {
+#pragma unroll 1
+            for (int p = g.t; p < npix; p += NT) {
+                int q0, q1, q2;
+                fix_split(fx, s[p], q0, q1, q2);
+                t0 += q0;
+                t1 += q1;
+                t2 += q2;
+                ++n;
+            }
         }
         tot = g.allsum_ll(fix_join(fx, t0 - n * kFixBias, t1 - n * kFixBias, t2 - n * kFixBias));
     }
