@@ -65,12 +65,9 @@ struct fse_ctx {
     cudaStream_t cls_stream[fse::kClasses - 1] = {};
     cudaEvent_t cls_fork = nullptr;
     cudaEvent_t cls_join[fse::kClasses - 1] = {};
-    // grow-only per-stamp coefficients of fse_moment_vjp, and growth-curve
-    // records of fse_moment_vjp / _jvp
+    // grow-only per-stamp coefficients of fse_moment_vjp
     fse::VjpCoef* d_vjp = nullptr;
     size_t vjp_cap = 0;
-    fse::R50Grad* d_r50 = nullptr;
-    size_t r50_cap = 0;
     // warps per CTA chosen by fse_autotune, by dtype, inverse variance and size
     // class (0 = library default)
     int tuned[2][2][fse::kClasses] = {};
@@ -515,7 +512,6 @@ void fse_destroy(fse_ctx* ctx) {
         cudaFree(ctx->d_perm);
         cudaFree(ctx->d_cls);
         cudaFree(ctx->d_vjp);
-        cudaFree(ctx->d_r50);
         for (int k = 0; k < fse::kClasses - 1; ++k) {
             if (ctx->cls_stream[k]) cudaStreamDestroy(ctx->cls_stream[k]);
             if (ctx->cls_join[k]) cudaEventDestroy(ctx->cls_join[k]);
@@ -1131,20 +1127,14 @@ static int moment_grad(fse_ctx* ctx, bool jvp, const void* pix, int dtype, const
     a.tangent = tangent;
     a.dtheta = dtheta;
     a.status = status;
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!jvp) {
-        // the analysis kernel's per-stamp coefficients for the write kernel
+        // the per-stamp coefficients for the write kernel
         const int rc = grow(ctx, &ctx->d_vjp, &ctx->vjp_cap, static_cast<size_t>(count));
         if (rc) return rc;
         a.coef = ctx->d_vjp;
     }
-    if (!jvp && (mode & FSE_MOM_SIGW_R50)) {
-        // the ring launch's growth-curve records for the analysis kernel
-        const int rc = grow(ctx, &ctx->d_r50, &ctx->r50_cap, static_cast<size_t>(count));
-        if (rc) return rc;
-        a.r50g = ctx->d_r50;
-    }
     a.queue = next_queue(ctx);
-    const cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "work counter reset");
     e = fse::launch_moment_grad(a, st);

@@ -12,8 +12,9 @@
 // so d theta / d I_p = -J^-1 W(p) m(p) with J_kl = sum_p I_p d(W m_k)/d theta_l.
 // Every m_k and every d R^2 / d theta_l is a polynomial of degree <= 2 in t,
 // so J is a fixed combination of the 15 weighted moments
-// M_ab = sum I W t1^a t2^b (a + b <= 4): one pass accumulates them, 25 lanes
-// assemble one entry of J each, and every lane solves the 5 x 5 system.
+// M_ab = sum I W t1^a t2^b (a + b <= 4).  A warp per stamp accumulates them,
+// assembles J with a lane per entry and solves the 5 x 5 system across its
+// lanes (moment_grad_kernel); for the VJP a streaming kernel then writes dL/dI.
 // sigma_w from the start-up growth curve (r50 / sqrt(2 ln 2), Sec. 4.1) is
 // an explicit function of the pixels: it is piecewise constant in the three
 // regions of the crossing ring (inside the disc k-1, in ring k, outside),
@@ -22,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "fse_device.cuh"
 #include "fse_internal.h"
@@ -34,15 +37,32 @@ constexpr float kInvSqrt2Ln2F = 0.849321800f;   // 1 / sqrt(2 ln 2)
 // Index of the monomial t1^a t2^b among the 15 of degree <= 4, by degree and
 // then by the power of t2.
 __host__ __device__ constexpr int mono(int a, int b) { return (a + b) * (a + b + 1) / 2 + b; }
-// The six monomials of degree <= 2: 1, t1, t2, t1^2, t1 t2, t2^2.
-__host__ __device__ constexpr int pa(int i) { return i == 1 || i == 3 || i == 4 ? (i == 3 ? 2 : 1) : 0; }
-__host__ __device__ constexpr int pb(int i) { return i == 2 || i == 4 || i == 5 ? (i == 5 ? 2 : 1) : 0; }
-
 template <int DT>
 __device__ __forceinline__ float load_pix(const MomentGradArgs& a, int64_t off, float sc) {
     return DT == FSE_BF16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(a.pix)[off]) * sc
                           : __ldg(static_cast<const float*>(a.pix) + off);
 }
+
+// The growth curve of the start-up (Sec. 4.1) around the brightest pixel, for
+// d sigma_w / d I: the crossing ring k (the first whose enclosed sum reaches
+// half the total) and the constants of d sigma_w / d I_p in the three regions
+// d <= k-1, k-1 < d <= k and d > k; for the JVP the tangent's sums over the
+// two discs.
+struct R50Grad {
+    int on;                  // sigma_w depends on the pixels
+    int pr, pc, k;
+    float c_in, c_ring, c_out;
+    float u_in, u_disc;      // JVP: tangent summed over d <= k-1 and d <= k
+};
+
+// A warp's sums of one stamp, in shared memory: the 15 weighted moments as
+// float pairs and the tangent's six weighted moments of degree <= 2 (JVP); and
+// the coefficient tables of the solve: the polynomials m_k and, in du, those of
+// d R^2 / d theta_l (l < 4) and R^2.
+struct MomSums {
+    float Mh[15], Ml[15], U[6];
+    float m[5][6], du[5][6];
+};
 
 // Stamp geometry at theta.
 struct Geom {
@@ -50,54 +70,20 @@ struct Geom {
     float A, B, G4, cw;      // R^2 = A t1^2 + B t2^2 - G4 t1 t2; W = 2^(cw R^2)
 };
 
-// Polynomial factors of degree <= 2 (coefficients of 1, t1, t2, t1^2, t1 t2,
-// t2^2) for J_kl = sum I W [a_l m_k + dm_k/dtheta_l]: m_k, a_l (the derivative
-// of log W: -R^2_l / 2 s^2, or R^2 / s^3 for sigma_w) and dm_k/dtheta_l.
-__device__ void jac_polys(const Geom& q, int k, int l, float mk[6], float al[6], float dm[6]) {
-    const float g1 = q.g1, g2 = q.g2, s = q.s, gg = g1 * g1 + g2 * g2;
-    const float ew1 = 2.f * g1 / (1.f + gg), ew2 = 2.f * g2 / (1.f + gg);
-    const float qq = (1.f + gg) * (1.f + gg);
-    const float dew[2][2] = {{2.f * (1.f - g1 * g1 + g2 * g2) / qq, -4.f * g1 * g2 / qq},
-                             {-4.f * g1 * g2 / qq, 2.f * (1.f + g1 * g1 - g2 * g2) / qq}};
-#pragma unroll
-    for (int i = 0; i < 6; ++i) mk[i] = al[i] = dm[i] = 0.f;
-    // d R^2 / d theta_l
-    float du[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (l == 0) { du[1] = -2.f * q.A; du[2] = q.G4; }
-    if (l == 1) { du[1] = q.G4; du[2] = -2.f * q.B; }
-    if (l == 2) { du[3] = 2.f * (g1 - 1.f); du[5] = 2.f * (g1 + 1.f); }
-    if (l == 3) { du[3] = 2.f * g2; du[4] = -4.f; du[5] = 2.f * g2; }
-    const float c = 1.f / (2.f * s * s);
-    if (l < 4) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) al[i] = -c * du[i];
-    } else {
-        const float is3 = 1.f / (s * s * s);
-        al[3] = q.A * is3; al[4] = -q.G4 * is3; al[5] = q.B * is3;
-    }
-    if (k == 0) { mk[1] = 1.f; if (l == 0) dm[0] = -1.f; }
-    if (k == 1) { mk[2] = 1.f; if (l == 1) dm[0] = -1.f; }
-    if (k == 2) {
-        mk[3] = 1.f - ew1; mk[5] = -(1.f + ew1);
-        if (l == 0) dm[1] = -2.f * (1.f - ew1);
-        if (l == 1) dm[2] = 2.f * (1.f + ew1);
-        if (l == 2 || l == 3) { dm[3] = dm[5] = -dew[0][l - 2]; }
-    }
-    if (k == 3) {
-        mk[3] = -ew2; mk[4] = 2.f; mk[5] = -ew2;
-        if (l == 0) { dm[1] = 2.f * ew2; dm[2] = -2.f; }
-        if (l == 1) { dm[1] = -2.f; dm[2] = 2.f * ew2; }
-        if (l == 2 || l == 3) { dm[3] = dm[5] = -dew[1][l - 2]; }
-    }
-    if (k == 4) {
-        mk[0] = -s * s; mk[3] = q.A; mk[4] = -q.G4; mk[5] = q.B;
-        if (l < 4) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) dm[i] = du[i];
-        } else {
-            dm[0] = -2.f * s;
-        }
-    }
+__device__ __forceinline__ Geom stamp_geom(const MomentGradArgs& a, const fse_result& mom) {
+    const bool ellip = (a.mode & FSE_MOM_ELLIP) != 0;
+    Geom q;
+    q.x0 = mom.x0;
+    q.y0 = mom.y0;
+    q.g1 = ellip ? mom.e1 : 0.f;
+    q.g2 = ellip ? mom.e2 : 0.f;
+    q.s = mom.sigma_w;
+    const float gg = q.g1 * q.g1 + q.g2 * q.g2;
+    q.A = 1.f + gg - 2.f * q.g1;
+    q.B = 1.f + gg + 2.f * q.g1;
+    q.G4 = 4.f * q.g2;
+    q.cw = -kLog2e / (2.f * q.s * q.s);
+    return q;
 }
 
 // Double-float helpers: the exact product error by FMA, Knuth's two-sum.
@@ -114,77 +100,121 @@ __device__ __forceinline__ void df_acc(float& hi, float& lo, float p, float e) {
     lo += err + e;
 }
 
-// One entry of J from the 15 moments (hi + lo pairs).  The combination
-// cancels by up to an order of magnitude (e.g. J_55 = sum I W [R^2 (R^2 - s^2)
-// / s^3 - 2 s]), so each coefficient, product and partial sum is carried in
-// double-float: once per stamp, 42 terms per lane.
-__device__ float jac_entry(const Geom& q, int k, int l, const float Mh[15], const float Ml[15]) {
-    float mk[6], al[6], dm[6];
-    jac_polys(q, k, l, mk, al, dm);
+// The polynomial factors of J (coefficients of 1, t1, t2, t1^2, t1 t2, t2^2)
+// into the warp's tables; the entries set here are the only ones that are ever
+// nonzero (the kernel clears the tables once).
+__device__ __forceinline__ void jac_tables(const Geom& q, int lane, MomSums* t) {
+    if (lane == 0) {
+        const float g1 = q.g1, g2 = q.g2, gg = g1 * g1 + g2 * g2;
+        const float ew1 = 2.f * g1 / (1.f + gg), ew2 = 2.f * g2 / (1.f + gg);
+        t->m[0][1] = 1.f;
+        t->m[1][2] = 1.f;
+        t->m[2][3] = 1.f - ew1; t->m[2][5] = -(1.f + ew1);
+        t->m[3][3] = -ew2; t->m[3][4] = 2.f; t->m[3][5] = -ew2;
+        t->m[4][0] = -q.s * q.s; t->m[4][3] = q.A; t->m[4][4] = -q.G4; t->m[4][5] = q.B;
+        t->du[0][1] = -2.f * q.A; t->du[0][2] = q.G4;
+        t->du[1][1] = q.G4; t->du[1][2] = -2.f * q.B;
+        t->du[2][3] = 2.f * (g1 - 1.f); t->du[2][5] = 2.f * (g1 + 1.f);
+        t->du[3][3] = 2.f * g2; t->du[3][4] = -4.f; t->du[3][5] = 2.f * g2;
+        t->du[4][3] = q.A; t->du[4][4] = -q.G4; t->du[4][5] = q.B;
+    }
+}
+
+// J_kl = sum I W [a_l m_k + dm_k/dtheta_l] from the 15 moments: with V[i] =
+// sum_j m_k[j] M_(i+j), J_kl = sum_i a_l[i] V[i] + sum_i dm_kl[i] M_i, where a_l
+// is the derivative of log W (-du_l / 2 s^2, or R^2 / s^3 for sigma_w) and
+// dm_k/dtheta_l follows from m_k: the centre moves t, so l = 0, 1 give -dm_k/dt1
+// and -dm_k/dt2; g enters m_3, m_4 through e_w and m_5 through R^2; sigma_w
+// enters m_5 alone.  The combination cancels by up to an order of magnitude
+// (e.g. J_55 = sum I W [R^2 (R^2 - s^2) / s^3 - 2 s]), so each product and
+// partial sum is carried in double-float.  One entry per lane.
+__device__ __forceinline__ float jac_entry(const Geom& q, const MomSums* t, int k, int l) {
+    const bool lin = l < 2;                 // a_l has the monomials t1, t2; else the squares
     float hi = 0.f, lo = 0.f;
+    {
+        const float* mk = t->m[k];
+        float c0 = 0.f, c1 = 0.f, c2 = 0.f; // dm_kl at 1, t1, t2 or at the squares
+        if (lin) {
+            c0 = -mk[1 + l];
+            c1 = l == 0 ? -2.f * mk[3] : -mk[4];
+            c2 = l == 0 ? -mk[4] : -2.f * mk[5];
+        } else if (k == 4) {
+            c0 = l < 4 ? t->du[l][3] : -2.f * q.s;
+            c1 = l < 4 ? t->du[l][4] : 0.f;
+            c2 = l < 4 ? t->du[l][5] : 0.f;
+        } else if (k >= 2 && l < 4) {
+            const float gg = q.g1 * q.g1 + q.g2 * q.g2, qq = (1.f + gg) * (1.f + gg);
+            const float d = q.g1 * q.g1 - q.g2 * q.g2;
+            const float de = k != l ? -4.f * q.g1 * q.g2 : 2.f * (k == 2 ? 1.f - d : 1.f + d);
+            c0 = c2 = -(de / qq);
+        }
+        const int b = l >= 2 && l < 4 ? 3 : 0;
+        const float c[3] = {c0, c1, c2};
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const int a = mono(pa(i), pb(i));
-        float p, e;
-        two_prod(dm[i], Mh[a], p, e);
-        df_acc(hi, lo, p, fmaf(dm[i], Ml[a], e));
+        for (int i = 0; i < 3; ++i) {
+            float p, e;
+            two_prod(c[i], t->Mh[b + i], p, e);
+            df_acc(hi, lo, p, fmaf(c[i], t->Ml[b + i], e));
+        }
+    }
+    const float fac = l < 4 ? -(1.f / (2.f * q.s * q.s)) : 1.f / (q.s * q.s * q.s);
+    const int n0 = lin ? 1 : 2;             // degree of a_l's monomials
+    const int tri[3] = {n0 * (n0 + 1) / 2, (n0 + 1) * (n0 + 2) / 2, (n0 + 2) * (n0 + 3) / 2};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {           // t1, t2 or t1^2, t1 t2, t2^2: power i of t2
+        const float a = lin && i == 2 ? 0.f : fac * t->du[l][(lin ? 1 : 3) + (lin && i == 2 ? 0 : i)];
+        float vh = 0.f, vl = 0.f, p, e;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-            const int b = mono(pa(i) + pa(j), pb(i) + pb(j));
-            float ch, cl;
-            two_prod(al[i], mk[j], ch, cl);
-            two_prod(ch, Mh[b], p, e);
-            df_acc(hi, lo, p, fmaf(ch, Ml[b], fmaf(cl, Mh[b], e)));
+            // degree and power of t2 of the j-th monomial
+            const int dj = j == 0 ? 0 : j < 3 ? 1 : 2, bj = j == 2 || j == 4 ? 1 : j == 5 ? 2 : 0;
+            const int b = lin && i == 2 ? 0 : tri[dj] + bj + i;
+            const float c = t->m[k][j];
+            two_prod(c, t->Mh[b], p, e);
+            df_acc(vh, vl, p, fmaf(c, t->Ml[b], e));
         }
+        two_prod(a, vh, p, e);
+        df_acc(hi, lo, p, fmaf(a, vl, e));
     }
     return hi + lo;
 }
 
-// Solve X x = r for 5 x 5 X (row-major) by Gaussian elimination with partial
-// pivoting, every index known at compile time.  Returns false if a pivot is
-// below 1e-6 of the largest entry.
-__device__ bool solve5(float X[25], float r[5], float x[5]) {
-    float big = 0.f;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) big = fmaxf(big, fabsf(X[i]));
+// Solve a 5 x 5 system held by 30 lanes, entry (r, c) in lane 6 r + c and the
+// right-hand side in column 5, by Gaussian elimination with partial pivoting
+// (rows are marked, not swapped).  Every lane gets the solution.  Returns
+// false if a pivot is below 1e-6 of `big`.
+__device__ __forceinline__ bool solve5(float X, float big, int lane, float (&x)[5]) {
+    const int r = lane / 6, c = lane - 6 * r;
+    unsigned done = 0;       // rows that have been pivots
+    int prow[5];             // pivot row of each column
     if (!(big > 0.f)) return false;
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
-        int piv = c;
-        float pv = fabsf(X[c * 5 + c]);
+    for (int s = 0; s < 5; ++s) {
+        float pv = -1.f, val = 0.f;
+        int piv = 0;
 #pragma unroll
-        for (int rr = c + 1; rr < 5; ++rr)
-            if (fabsf(X[rr * 5 + c]) > pv) { pv = fabsf(X[rr * 5 + c]); piv = rr; }
-        if (!(pv > 1e-6f * big)) return false;
-#pragma unroll
-        for (int rr = c + 1; rr < 5; ++rr) {
-            if (rr == piv) {
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    const float t = X[c * 5 + k];
-                    X[c * 5 + k] = X[rr * 5 + k];
-                    X[rr * 5 + k] = t;
-                }
-                const float t = r[c];
-                r[c] = r[rr];
-                r[rr] = t;
+        for (int i = 0; i < 5; ++i) {
+            const float v = __shfl_sync(kFull, X, 6 * i + s);
+            if (!(done >> i & 1) && fabsf(v) > pv) {
+                pv = fabsf(v);
+                val = v;
+                piv = i;
             }
         }
-        const float inv = 1.f / X[c * 5 + c];
-#pragma unroll
-        for (int rr = c + 1; rr < 5; ++rr) {
-            const float f = X[rr * 5 + c] * inv;
-#pragma unroll
-            for (int k = c; k < 5; ++k) X[rr * 5 + k] = fmaf(-f, X[c * 5 + k], X[rr * 5 + k]);
-            r[rr] = fmaf(-f, r[c], r[rr]);
-        }
+        if (!(pv > 1e-6f * big)) return false;
+        const float inv = 1.f / val;
+        const float mine = __shfl_sync(kFull, X, 6 * (r < 5 ? r : 0) + s);
+        const float row = __shfl_sync(kFull, X, 6 * piv + c);
+        done |= 1u << piv;
+        prow[s] = piv;
+        if (!(done >> r & 1)) X = fmaf(-(mine * inv), row, X);
     }
 #pragma unroll
-    for (int rr = 4; rr >= 0; --rr) {
-        float acc = r[rr];
+    for (int s = 4; s >= 0; --s) {
+        float acc = __shfl_sync(kFull, X, 6 * prow[s] + 5);
 #pragma unroll
-        for (int k = rr + 1; k < 5; ++k) acc = fmaf(-X[rr * 5 + k], x[k], acc);
-        x[rr] = acc / X[rr * 5 + rr];
+        for (int j = s + 1; j < 5; ++j) acc = fmaf(-__shfl_sync(kFull, X, 6 * prow[s] + j), x[j], acc);
+        x[s] = acc / __shfl_sync(kFull, X, 6 * prow[s] + s);
     }
     return true;
 }
@@ -196,9 +226,11 @@ __device__ bool solve5(float X[25], float r[5], float x[5]) {
 // start-up's own except where an enclosed sum lies within ~1e-13 of half the
 // total.  For the JVP the tangent's sums over the two discs come with them.
 
+// Only the square that holds the disc is read (from L1 or L2: the stamp was
+// read just before).
 template <int DT, bool JVP>
-__device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, int npix, float sc, float r50_hint,
-                            int peak, float tot_h, float tot_l, int lane) {
+__device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, float sc, float r50_hint, int peak,
+                            float tot_h, float tot_l, int lane) {
     R50Grad o;
     o.on = 0;
     o.pr = peak / ix.w;
@@ -209,28 +241,33 @@ __device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, int np
     if (!(tot > 0.f)) return o;                  // fallback radius: no dependence
     // candidate from the start-up radius: r50 = (k-1) + frac, frac in (0, 1]
     int k = r50_hint > 0.5f ? static_cast<int>(ceilf(r50_hint)) : 0;
+#pragma unroll 1
     for (int tries = 0; tries < 8; ++tries) {
         float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
         const float km2 = static_cast<float>((k - 1) * (k - 1)), k2 = static_cast<float>(k * k);
-        const float pcf = static_cast<float>(o.pc), prf = static_cast<float>(o.pr);
-        FWalk pw(lane, ix.w);
-        int p0 = lane;
-        for (; p0 < npix; p0 += 256) {
-            // eight loads in flight per lane; the stamp is still in L1 or L2
-            float v[8], uu[8];
+        Box bx;
+        bx.r0 = max(0, o.pr - k);
+        bx.c0 = max(0, o.pc - k);
+        bx.bh = min(ix.h - 1, o.pr + k) - bx.r0 + 1;
+        bx.bw = min(ix.w - 1, o.pc + k) - bx.c0 + 1;
+        const int plast = bx.last(ix.w);
+        BoxWalk bk(lane, bx, ix.w, 32, o.pc, o.pr);
+#pragma unroll 1
+        while (__any_sync(kFull, bk.p <= plast)) {
+            // four loads in flight per lane
+            float v[4], uu[4], d2[4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int p = p0 + 32 * u;
-                v[u] = p < npix ? load_pix<DT>(a, ix.offset + p, sc) : 0.f;
-                if (JVP) uu[u] = p < npix ? __ldg(a.tangent + ix.offset + p) : 0.f;
+            for (int u = 0; u < 4; ++u) {
+                const bool in = bk.p <= plast;
+                v[u] = in ? load_pix<DT>(a, ix.offset + bk.p, sc) : 0.f;
+                if (JVP) uu[u] = in ? __ldg(a.tangent + ix.offset + bk.p) : 0.f;
+                d2[u] = fmaf(bk.v, bk.v, bk.u * bk.u);       // an exact integer
+                bk.next();
             }
             float ph[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float dj = pw.c - pcf, di = pw.r - prf;
-                const float d2 = fmaf(di, di, dj * dj);      // an exact integer
-                pw.next();
-                const bool in0 = k >= 1 && d2 <= km2, in1 = d2 <= k2;   // zero-filled past the end
+            for (int u = 0; u < 4; ++u) {
+                const bool in0 = k >= 1 && d2[u] <= km2, in1 = d2[u] <= k2;   // zero-filled past the end
                 ph[0] += in0 ? v[u] : 0.f;
                 ph[1] += in1 ? v[u] : 0.f;
                 if (JVP) {
@@ -239,9 +276,15 @@ __device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, int np
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) df_add(h[i], l[i], ph[i]);
+            for (int i = 0; i < (JVP ? 4 : 2); ++i) df_add(h[i], l[i], ph[i]);
         }
-        warp_allsum_df(h, l);
+        if constexpr (JVP) {
+            warp_allsum_df(h, l);
+        } else {
+            float h2[2] = {h[0], h[1]}, l2[2] = {l[0], l[1]};
+            warp_allsum_df(h2, l2);
+            h[0] = h2[0]; h[1] = h2[1]; l[0] = l2[0]; l[1] = l2[1];
+        }
         // 2 E - tot in double-float: the sign decides the crossing
         const float d1 = (2.f * h[1] - tot_h) + (2.f * l[1] - tot_l);
         const float d0 = (2.f * h[0] - tot_h) + (2.f * l[0] - tot_l);
@@ -275,10 +318,10 @@ __device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, int np
 
 // The moment terms of one pixel at t = (t1, t2): f = I W times the 15
 // monomials of degree <= 4 into P; for the JVP, the tangent u W times the
-// six of degree <= 2, and u itself, into PU.
+// six of degree <= 2 into PU.
 template <bool JVP>
 __device__ __forceinline__ void moment_terms(const Geom& q, float t1, float t2, float v, float uu, float (&P)[15],
-                                             float (&PU)[7]) {
+                                             float (&PU)[6]) {
     const float R2 = fmaf(q.A, t1 * t1, fmaf(q.B, t2 * t2, -q.G4 * (t1 * t2)));
     const float W = ex2(R2 * q.cw);
     const float f = v * W;
@@ -309,86 +352,103 @@ __device__ __forceinline__ void moment_terms(const Geom& q, float t1, float t2, 
         PU[3] = fmaf(h1, t1, PU[3]);
         PU[4] = fmaf(h1, t2, PU[4]);
         PU[5] = fmaf(h2, t2, PU[5]);
-        PU[6] += uu;
     }
 }
 
-// One warp per stamp.  JVP = true: dtheta along a.tangent; false: the pixel
-// gradient for a.v.
+// The weighted sums of one stamp, by one warp, in one pass over its pixels
+// (eight loads in flight per lane): finiteness; with sigma_w from the growth
+// curve the brightest pixel and the total; for the JVP the tangent's total;
+// and, where the rows of a block of 256 pixels meet the weight's box (W >=
+// 2^-40, weight_box; the rest adds less than 2^-40 |I| |t|^4 to a sum), the 15
+// weighted moments and, for the JVP, the tangent's six: eight pixels per lane
+// in fp32, then double-float.  Then the growth curve's crossing ring
+// (r50_ring).  The totals go to rec from the lanes that hold them after the
+// exchange.  (A second pass over the box's pixels alone has a third fewer
+// weights to evaluate, but its walk and its wait for the loads cost more.)
 template <int DT, bool JVP>
-__global__ void __launch_bounds__(256, 2) moment_grad_kernel(MomentGradArgs a) {
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned sidx = 0;
-        if (lane == 0) sidx = atomicAdd(a.queue, 1u);
-        sidx = __shfl_sync(kFull, sidx, 0);
-        if (sidx >= static_cast<unsigned long long>(a.count)) break;
-        const int64_t si = static_cast<int64_t>(sidx);
-        const fse_stamp ix = a.idx[si];
-        const fse_result mom = a.moments[si];
-        uint32_t status = 0;
-        const long long npl = static_cast<long long>(ix.h) * ix.w;
-        if (ix.h < 1 || ix.w < 1 || npl > FSE_MAX_PIX) {
-            if (lane == 0 && a.status) a.status[si] = FSE_ST_BAD_SIZE;
-            if (JVP && lane < 5) a.dtheta[si * 5 + lane] = 0.f;
-            continue;
-        }
+__device__ __forceinline__ void stamp_grad(const MomentGradArgs& a, int64_t si, int lane, MomSums* rec) {
+    const fse_stamp ix = a.idx[si];
+    const fse_result mom = a.moments[si];
+    const long long npl = static_cast<long long>(ix.h) * ix.w;
+    uint32_t status = 0;
+    R50Grad rg;
+    rg.on = 0;
+    rg.pr = rg.pc = rg.k = 0;
+    rg.c_in = rg.c_ring = rg.c_out = rg.u_in = rg.u_disc = 0.f;
+    float dsw = 0.f;
+    const Geom q = stamp_geom(a, mom);
+    const bool ellip = (a.mode & FSE_MOM_ELLIP) != 0;
+    const bool sig_held = (a.mode & FSE_MOM_SIGW_FIXED) || (mom.status & FSE_ST_SIGW_CLAMPED);
+    const bool sig_r50 = !sig_held && (a.mode & FSE_MOM_SIGW_R50);
+    if (ix.h < 1 || ix.w < 1 || npl > FSE_MAX_PIX) {
+        status = FSE_ST_BAD_SIZE;
+    } else {
         const int npix = static_cast<int>(npl);
         if (!(mom.status & FSE_ST_MOM_CONVERGED)) status |= FSE_ST_MOM_FAILED;
-        const bool ellip = (a.mode & FSE_MOM_ELLIP) != 0;
-        const bool sig_held = (a.mode & FSE_MOM_SIGW_FIXED) || (mom.status & FSE_ST_SIGW_CLAMPED);
-        const bool sig_r50 = !sig_held && (a.mode & FSE_MOM_SIGW_R50);
-        const float sc = (DT == FSE_BF16 && a.scale) ? a.scale[si] : 1.f;
-        Geom q;
-        q.x0 = mom.x0;
-        q.y0 = mom.y0;
-        q.g1 = ellip ? mom.e1 : 0.f;
-        q.g2 = ellip ? mom.e2 : 0.f;
-        q.s = mom.sigma_w;
-        {
-            const float gg = q.g1 * q.g1 + q.g2 * q.g2;
-            q.A = 1.f + gg - 2.f * q.g1;
-            q.B = 1.f + gg + 2.f * q.g1;
-            q.G4 = 4.f * q.g2;
-            q.cw = -kLog2e / (2.f * q.s * q.s);
-        }
         if (!(q.s > 0.f) || !isfinite(q.cw)) status |= FSE_ST_MOM_FAILED;
-        bool finite = true;
-        // pass 1: the 15 weighted moments; the tangent's weighted sums (JVP);
-        // and, for the growth curve, the brightest pixel and the total
-        float Mh[15], Ml[15], Uh[7], Ul[7];
-#pragma unroll
-        for (int i = 0; i < 15; ++i) Mh[i] = Ml[i] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 7; ++i) Uh[i] = Ul[i] = 0.f;
-        // JVP: the brightest pixel and the total ride along the moments pass
-        // (its one launch reads the stamp once); the VJP has them from the
-        // ring launch
-        const bool inl = JVP && sig_r50;
-        float vmax = -INFINITY, th_ = 0.f, tl_ = 0.f;
-        int imax = 0x7fffffff;
+        const float sc = (DT == FSE_BF16 && a.scale) ? a.scale[si] : 1.f;
         if (status == 0) {
+            float vmax = -INFINITY, zero = 0.f;
+            int imax = 0x7fffffff;
+            float th[2] = {0.f, 0.f}, tl[2] = {0.f, 0.f};   // totals of the pixels and of the tangent
+            float Mh[15], Ml[15], Uh[6], Ul[6];
+#pragma unroll
+            for (int i = 0; i < 15; ++i) Mh[i] = Ml[i] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) Uh[i] = Ul[i] = 0.f;
+            // the pixels of the box's rows
+            const Box bx = weight_box(q.x0, q.y0, q.g1, q.g2, q.s, ix.h, ix.w);
+            const int box0 = bx.r0 * ix.w, box1 = (bx.r0 + bx.bh) * ix.w;
             FWalk pw(lane, ix.w);
-            int p0 = lane;
-            // eight pixels per lane per step, loads ahead of use; then the tail
-            for (; p0 + 224 < npix; p0 += 256) {
-                float P[15], PU[7], ptot = 0.f;
-#pragma unroll
-                for (int i = 0; i < 15; ++i) P[i] = 0.f;
-#pragma unroll
-                for (int i = 0; i < 7; ++i) PU[i] = 0.f;
+#pragma unroll 1
+            for (int b0 = 0; b0 < npix; b0 += 256) {
                 float v[8], uu[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    v[u] = load_pix<DT>(a, ix.offset + p0 + 32 * u, sc);
-                    if (JVP) uu[u] = __ldg(a.tangent + ix.offset + p0 + 32 * u);
+                    const int p = b0 + 32 * u + lane;
+                    v[u] = p < npix ? load_pix<DT>(a, ix.offset + p, sc) : 0.f;
+                    if (JVP) uu[u] = p < npix ? __ldg(a.tangent + ix.offset + p) : 0.f;
                 }
+                float pt = 0.f, pu = 0.f;
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    if (JVP && inl) {
-                        if (v[u] > vmax) { vmax = v[u]; imax = p0 + 32 * u; }
-                        ptot += v[u];
+                    zero = fmaf(v[u], 0.f, zero);   // NaN from a NaN or infinite pixel
+                    pt += v[u];
+                    if (JVP) pu += uu[u];
+                }
+                if (sig_r50) {
+                    // the lane's maximum of the eight, and its index where it leads
+                    float m8 = v[0];
+                    if (b0 + 256 <= npix) {
+#pragma unroll
+                        for (int u = 1; u < 8; ++u) m8 = fmaxf(m8, v[u]);
+                    } else {
+                        m8 = -INFINITY;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) m8 = b0 + 32 * u + lane < npix ? fmaxf(m8, v[u]) : m8;
                     }
+                    if (m8 > vmax) {
+                        vmax = m8;
+#pragma unroll
+                        for (int u = 7; u >= 0; --u)
+                            if (v[u] == m8 && b0 + 32 * u + lane < npix) imax = b0 + 32 * u + lane;
+                    }
+                    df_add(th[0], tl[0], pt);
+                }
+                if (JVP) df_add(th[1], tl[1], pu);
+                if (b0 + 256 <= box0 || b0 >= box1) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) pw.next();
+                    continue;
+                }
+                float P[15], PU[6];
+#pragma unroll
+                for (int i = 0; i < 15; ++i) P[i] = 0.f;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) PU[i] = 0.f;
+                // (pixels past the end are zero and add nothing)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
                     moment_terms<JVP>(q, pw.c - q.x0, pw.r - q.y0, v[u], JVP ? uu[u] : 0.f, P, PU);
                     pw.next();
                 }
@@ -396,253 +456,167 @@ __global__ void __launch_bounds__(256, 2) moment_grad_kernel(MomentGradArgs a) {
                 for (int i = 0; i < 15; ++i) df_add(Mh[i], Ml[i], P[i]);
                 if (JVP) {
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) df_add(Uh[i], Ul[i], PU[i]);
-                    if (inl) df_add(th_, tl_, ptot);
+                    for (int i = 0; i < 6; ++i) df_add(Uh[i], Ul[i], PU[i]);
                 }
             }
-            {
-                float P[15], PU[7], ptot = 0.f;
-#pragma unroll
-                for (int i = 0; i < 15; ++i) P[i] = 0.f;
-#pragma unroll
-                for (int i = 0; i < 7; ++i) PU[i] = 0.f;
-                for (int p = p0; p < npix; p += 32) {
-                    const float v = load_pix<DT>(a, ix.offset + p, sc);
-                    const float uu = JVP ? __ldg(a.tangent + ix.offset + p) : 0.f;
-                    if (JVP && inl) {
-                        if (v > vmax) { vmax = v; imax = p; }
-                        ptot += v;
-                    }
-                    moment_terms<JVP>(q, pw.c - q.x0, pw.r - q.y0, v, uu, P, PU);
-                    pw.next();
-                }
-#pragma unroll
-                for (int i = 0; i < 15; ++i) df_add(Mh[i], Ml[i], P[i]);
-                if (JVP) {
-#pragma unroll
-                    for (int i = 0; i < 7; ++i) df_add(Uh[i], Ul[i], PU[i]);
-                    if (inl) df_add(th_, tl_, ptot);
-                }
+            scatter_sum_df<15, 16>(Mh, Ml, lane);
+            const int j = scatter_index<15>(lane);
+            if (j < 15) {
+                rec->Mh[j] = Mh[0];
+                rec->Ml[j] = Ml[0];
             }
-            // a NaN or Inf pixel (or tangent) makes I W (u W) non-finite
-            // whatever its weight, and with it the warp's total
-            float chk = (Mh[0] + Ml[0]) + (JVP ? Uh[6] + Uh[0] : 0.f) + (inl ? th_ : 0.f);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) chk += __shfl_xor_sync(kFull, chk, off);
-            finite = isfinite(chk);
-        }
-        if (!finite) status |= FSE_ST_NONFINITE;
-        float Su[7];
-        if (status == 0) {
-            warp_allsum_df(Mh, Ml);
             if (JVP) {
-                warp_allsum_df(Uh, Ul);
-#pragma unroll
-                for (int i = 0; i < 7; ++i) Su[i] = Uh[i] + Ul[i];
+                scatter_sum_df<6, 16>(Uh, Ul, lane);
+                const int i = scatter_index<6>(lane);
+                if (i < 6) rec->U[i] = Uh[0] + Ul[0];
             }
-        }
-        // the growth curve's crossing ring and constants, from the ring launch
-        R50Grad rg;
-        rg.on = 0;
-        rg.pr = rg.pc = rg.k = 0;
-        rg.c_in = rg.c_ring = rg.c_out = rg.u_in = rg.u_disc = 0.f;
-        if (status == 0 && sig_r50) {
-            if constexpr (JVP) {
+            if (sig_r50) {
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
                     const float ov = __shfl_xor_sync(kFull, vmax, off);
                     const int oi = __shfl_xor_sync(kFull, imax, off);
                     if (ov > vmax || (ov == vmax && oi < imax)) { vmax = ov; imax = oi; }
                 }
-                float t2h[1] = {th_}, t2l[1] = {tl_};
-                warp_allsum_df(t2h, t2l);
-                rg = r50_ring<DT, JVP>(a, ix, npix, sc, mom.r50, imax, t2h[0], t2l[0], lane);
-            } else {
-                rg = a.r50g[si];
+            }
+            if (JVP || sig_r50) warp_allsum_df(th, tl);
+            float chk = zero;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) chk += __shfl_xor_sync(kFull, chk, off);
+            if (JVP) chk += th[1] + (sig_r50 ? th[0] : 0.f);
+            if (!isfinite(chk)) status |= FSE_ST_NONFINITE;
+            if (status == 0 && sig_r50 && isfinite(th[0])) {
+                rg = r50_ring<DT, JVP>(a, ix, sc, mom.r50, imax, th[0], tl[0], lane);
+                if (JVP && rg.on)
+                    dsw = rg.c_out * (th[1] + tl[1]) + (rg.c_ring - rg.c_out) * rg.u_disc +
+                          (rg.c_in - rg.c_ring) * rg.u_in;
             }
         }
-        // J: lane 5k + l assembles J_kl; then every lane holds all 25
-        float X[25], xs[5], rhs[5];
-        bool solved = false;
-        float Jcol4[5];
-        if (status == 0) {
-            const int k = lane < 25 ? lane / 5 : 0, l = lane < 25 ? lane - 5 * (lane / 5) : 0;
-            const float mine = jac_entry(q, k, l, Mh, Ml);
-#pragma unroll
-            for (int i = 0; i < 25; ++i) X[i] = __shfl_sync(kFull, mine, i);
-#pragma unroll
-            for (int i = 0; i < 5; ++i) Jcol4[i] = X[i * 5 + 4];
-            // held parameters: rows and columns of a diagonal entry as large
-            // as the active block's largest, with a zero right-hand side
-            bool act[5] = {true, true, ellip, ellip, !(sig_held || sig_r50)};
-            float big = 0.f;
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-#pragma unroll
-                for (int j = 0; j < 5; ++j)
-                    if (act[i] && act[j]) big = fmaxf(big, fabsf(X[i * 5 + j]));
-#pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                if (!act[i]) {
-#pragma unroll
-                    for (int j = 0; j < 5; ++j) X[i * 5 + j] = X[j * 5 + i] = 0.f;
-                    X[i * 5 + i] = big;
-                }
-            }
-            if (JVP) {
-                // rhs = -(sum u psi + J_as dsigma_w); psi_k = W m_k
-                float dsw = 0.f;
-                if (rg.on)
-                    dsw = rg.c_out * Su[6] + (rg.c_ring - rg.c_out) * rg.u_disc + (rg.c_in - rg.c_ring) * rg.u_in;
-                const float ew1 = 2.f * q.g1 / (1.f + q.g1 * q.g1 + q.g2 * q.g2);
-                const float ew2 = 2.f * q.g2 / (1.f + q.g1 * q.g1 + q.g2 * q.g2);
-                float S5[5];
-                S5[0] = Su[1];
-                S5[1] = Su[2];
-                S5[2] = (1.f - ew1) * Su[3] - (1.f + ew1) * Su[5];
-                S5[3] = 2.f * Su[4] - ew2 * (Su[3] + Su[5]);
-                S5[4] = q.A * Su[3] - q.G4 * Su[4] + q.B * Su[5] - q.s * q.s * Su[0];
-#pragma unroll
-                for (int i = 0; i < 5; ++i) rhs[i] = act[i] ? -(S5[i] + Jcol4[i] * dsw) : 0.f;
-                solved = solve5(X, rhs, xs);
-                if (solved && rg.on) xs[4] = dsw;
-            } else {
-                // transpose for J^T lambda = v
-#pragma unroll
-                for (int i = 0; i < 5; ++i)
-#pragma unroll
-                    for (int j = i + 1; j < 5; ++j) {
-                        const float t = X[i * 5 + j];
-                        X[i * 5 + j] = X[j * 5 + i];
-                        X[j * 5 + i] = t;
-                    }
-#pragma unroll
-                for (int i = 0; i < 5; ++i) rhs[i] = act[i] ? a.v[si * 5 + i] : 0.f;
-                solved = solve5(X, rhs, xs);
-            }
-            if (!solved) status |= FSE_ST_FIT_SINGULAR;
-        }
-        if (JVP) {
-            float val = 0.f;
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-                if (lane == i && status == 0) val = xs[i];
-            if (lane < 5) a.dtheta[si * 5 + lane] = val;
-        } else {
-            // dL/dI_p = -W(p) sum_k lambda_k m_k(p) + kappa d sigma_w / d I_p:
-            // the per-stamp coefficients, for the write kernel
-            VjpCoef cf;
-            cf.x0 = q.x0;
-            cf.y0 = q.y0;
-            cf.A = q.A;
-            cf.B = q.B;
-            cf.G4 = q.G4;
-            cf.cw = q.cw;
-#pragma unroll
-            for (int i = 0; i < 6; ++i) cf.c[i] = 0.f;
-            cf.kc_in = cf.kc_ring = cf.kc_out = 0.f;
-            cf.pc = static_cast<float>(rg.pc);
-            cf.pr = static_cast<float>(rg.pr);
-            cf.km2 = rg.k >= 1 ? static_cast<float>((rg.k - 1) * (rg.k - 1)) : -1.f;
-            cf.k2 = static_cast<float>(rg.k * rg.k);
-            cf.ring = rg.on && status == 0;
-            cf.ok = status == 0;
-            if (status == 0) {
-                const float gg = q.g1 * q.g1 + q.g2 * q.g2;
-                const float ew1 = 2.f * q.g1 / (1.f + gg), ew2 = 2.f * q.g2 / (1.f + gg);
-                cf.c[0] = -xs[4] * q.s * q.s;
-                cf.c[1] = xs[0];
-                cf.c[2] = xs[1];
-                cf.c[3] = xs[2] * (1.f - ew1) - xs[3] * ew2 + xs[4] * q.A;
-                cf.c[4] = 2.f * xs[3] - xs[4] * q.G4;
-                cf.c[5] = -xs[2] * (1.f + ew1) - xs[3] * ew2 + xs[4] * q.B;
-                if (rg.on) {
-                    float kappa = a.v[si * 5 + 4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) kappa = fmaf(-xs[i], Jcol4[i], kappa);
-                    cf.kc_in = kappa * rg.c_in;
-                    cf.kc_ring = kappa * rg.c_ring;
-                    cf.kc_out = kappa * rg.c_out;
-                }
-            }
-            if (lane == 0) a.coef[si] = cf;
-        }
-        if (lane == 0 && a.status) a.status[si] = status;
     }
+    // J, a lane per entry, and the solve
+    float xs[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Jcol4[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    if (status == 0) {
+        jac_tables(q, lane, rec);
+        __syncwarp();   // the sums and the tables are in place
+        if (!isfinite(rec->Mh[0] + rec->Ml[0] + (JVP ? rec->U[0] : 0.f))) status |= FSE_ST_NONFINITE;
+    }
+    if (status == 0) {
+        // lane 6 r + c: entry (r, c) of J (JVP) or of its transpose (VJP), the
+        // right-hand side in column 5
+        const int r = lane < 30 ? lane / 6 : 0, c = lane < 30 ? lane - 6 * (lane / 6) : 0;
+        const int k = JVP || c == 5 ? r : c, l = c == 5 ? 4 : (JVP ? c : r);
+        float X = jac_entry(q, rec, k, l);      // column 5: J_r4, for the coupling to sigma_w
+        // lane of J_i4: (i, 4), or (4, i) in the transpose
+#pragma unroll
+        for (int i = 0; i < 5; ++i) Jcol4[i] = __shfl_sync(kFull, X, JVP ? 6 * i + 4 : 24 + i);
+        // held parameters: rows and columns of a diagonal entry as large as the
+        // active block's largest, with a zero right-hand side
+        const unsigned act = 3u | (ellip ? 12u : 0u) | (sig_held || sig_r50 ? 0u : 16u);
+        const bool on = (act >> k & 1) && (act >> l & 1) && c < 5 && lane < 30;
+        const float big = __uint_as_float(__reduce_max_sync(kFull, on ? __float_as_uint(fabsf(X)) : 0u));
+        if (c == 5) {
+            float rv;
+            if (JVP) {
+                // -(sum u psi + J_as dsigma_w); psi_k = W m_k
+                float S5 = 0.f;
+#pragma unroll
+                for (int j = 5; j >= 0; --j) S5 = fmaf(rec->m[r][j], rec->U[j], S5);
+                rv = -(S5 + X * dsw);
+            } else {
+                rv = a.v[si * 5 + r];
+            }
+            X = (act >> r & 1) ? rv : 0.f;
+        } else if (!on) {
+            X = r == c ? big : 0.f;
+        }
+        if (!solve5(X, big, lane, xs)) status |= FSE_ST_FIT_SINGULAR;
+    }
+    if (JVP) {
+        float val = 0.f;
+        if (rg.on) xs[4] = dsw;
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+            if (lane == i && status == 0) val = xs[i];
+        if (lane < 5) a.dtheta[si * 5 + lane] = val;
+    } else if (lane == 0) {
+        // dL/dI_p = -W(p) sum_k lambda_k m_k(p) + kappa d sigma_w / d I_p:
+        // the per-stamp coefficients, for the write kernel
+        VjpCoef cf;
+        cf.x0 = q.x0;
+        cf.y0 = q.y0;
+        cf.A = q.A;
+        cf.B = q.B;
+        cf.G4 = q.G4;
+        cf.cw = q.cw;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) cf.c[i] = 0.f;
+        cf.kc_in = cf.kc_ring = cf.kc_out = 0.f;
+        cf.pc = static_cast<float>(rg.pc);
+        cf.pr = static_cast<float>(rg.pr);
+        cf.km2 = rg.k >= 1 ? static_cast<float>((rg.k - 1) * (rg.k - 1)) : -1.f;
+        cf.k2 = static_cast<float>(rg.k * rg.k);
+        cf.ring = rg.on && status == 0;
+        cf.ok = status == 0;
+        if (status == 0) {
+            const float gg = q.g1 * q.g1 + q.g2 * q.g2;
+            const float ew1 = 2.f * q.g1 / (1.f + gg), ew2 = 2.f * q.g2 / (1.f + gg);
+            cf.c[0] = -xs[4] * q.s * q.s;
+            cf.c[1] = xs[0];
+            cf.c[2] = xs[1];
+            cf.c[3] = xs[2] * (1.f - ew1) - xs[3] * ew2 + xs[4] * q.A;
+            cf.c[4] = 2.f * xs[3] - xs[4] * q.G4;
+            cf.c[5] = -xs[2] * (1.f + ew1) - xs[3] * ew2 + xs[4] * q.B;
+            if (rg.on) {
+                float kappa = a.v[si * 5 + 4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) kappa = fmaf(-xs[i], Jcol4[i], kappa);
+                cf.kc_in = kappa * rg.c_in;
+                cf.kc_ring = kappa * rg.c_ring;
+                cf.kc_out = kappa * rg.c_out;
+            }
+        }
+        a.coef[si] = cf;
+    }
+    if (lane == 0 && a.status) a.status[si] = status;
+    __syncwarp();   // the sums have been read
 }
 
-// The growth curve of the start-up for the VJP's sigma_w derivative, in a
-// launch of its own (the analysis kernel's body is long enough that its warps
-// wait on instruction fetch; the JVP keeps it in its one kernel, whose passes
-// then read the stamp from DRAM once): per stamp, one pass for the brightest
-// pixel (ties to the lowest index) and the double-float total, then
-// r50_ring's disc sums; the record goes to a.r50g for the analysis kernel.  One warp per stamp, stamps
-// in grid-stride order; a stamp whose sigma_w does not come from the growth
-// curve, or that the analysis kernel skips, gets on = 0.
+// One warp per stamp, from the work counter.
+//   50,000 stamps of 48x48 (JVP, sigma_w from the growth curve; 922 MB read,
+//   0.136 ms at the copy rate): 0.87 ms with the ring's disc sums over the whole
+//   stamp, a generic 42-term entry of J per lane and the 5 x 5 solve repeated in
+//   every lane; 0.73 ms with the warp sums by exchange; 0.56 ms as it is, bound by
+//   issue and instruction fetch (2,000 instructions outside the pixel loop).  A
+//   lane per stamp for the solve, 32 stamps at a time, took 0.42 ms here but 75
+//   instead of 53 us at 2,090 stamps of 62x62, where it fetches its code for one
+//   stamp per warp.
 template <int DT, bool JVP>
-__global__ void __launch_bounds__(256) moment_r50_kernel(MomentGradArgs a) {
+__global__ void __launch_bounds__(256, 2) moment_grad_kernel(MomentGradArgs a) {
+    __shared__ MomSums s_rec[8];
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    for (int64_t si = gw; si < a.count; si += nw) {
-        const fse_stamp ix = a.idx[si];
-        const fse_result mom = a.moments[si];
-        R50Grad rg;
-        rg.on = 0;
-        rg.pr = rg.pc = rg.k = 0;
-        rg.c_in = rg.c_ring = rg.c_out = rg.u_in = rg.u_disc = 0.f;
-        const long long npl = static_cast<long long>(ix.h) * ix.w;
-        const bool sig_held = (a.mode & FSE_MOM_SIGW_FIXED) || (mom.status & FSE_ST_SIGW_CLAMPED);
-        const bool use = ix.h >= 1 && ix.w >= 1 && npl <= FSE_MAX_PIX && (mom.status & FSE_ST_MOM_CONVERGED) &&
-                         !sig_held && (a.mode & FSE_MOM_SIGW_R50);
-        if (use) {
-            const int npix = static_cast<int>(npl);
-            const float sc = (DT == FSE_BF16 && a.scale) ? a.scale[si] : 1.f;
-            float vmax = -INFINITY;
-            int imax = 0x7fffffff;
-            float th[1] = {0.f}, tl[1] = {0.f};
-            int p0 = lane;
-            for (; p0 + 224 < npix; p0 += 256) {
-                float v[8], pt = 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = load_pix<DT>(a, ix.offset + p0 + 32 * u, sc);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (v[u] > vmax) { vmax = v[u]; imax = p0 + 32 * u; }
-                    pt += v[u];
-                }
-                df_add(th[0], tl[0], pt);
-            }
-            {
-                float pt = 0.f;
-                for (int p = p0; p < npix; p += 32) {
-                    const float v = load_pix<DT>(a, ix.offset + p, sc);
-                    if (v > vmax) { vmax = v; imax = p; }
-                    pt += v;
-                }
-                df_add(th[0], tl[0], pt);
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const float ov = __shfl_xor_sync(kFull, vmax, off);
-                const int oi = __shfl_xor_sync(kFull, imax, off);
-                if (ov > vmax || (ov == vmax && oi < imax)) { vmax = ov; imax = oi; }
-            }
-            warp_allsum_df(th, tl);
-            // a non-finite pixel leaves the total non-finite: no dependence
-            // (the analysis kernel flags the stamp)
-            if (isfinite(th[0]) && imax < npix)
-                rg = r50_ring<DT, JVP>(a, ix, npix, sc, mom.r50, imax, th[0], tl[0], lane);
-        }
-        if (lane == 0) a.r50g[si] = rg;
+    MomSums* rec = &s_rec[threadIdx.x >> 5];
+    if (lane < 30) {
+        rec->m[lane / 6][lane % 6] = 0.f;
+        rec->du[lane / 6][lane % 6] = 0.f;
+    }
+    __syncwarp();
+    for (;;) {
+        unsigned sidx = 0;
+        if (lane == 0) sidx = atomicAdd(a.queue, 1u);
+        sidx = __shfl_sync(kFull, sidx, 0);
+        if (sidx >= static_cast<unsigned long long>(a.count)) break;
+        stamp_grad<DT, JVP>(a, static_cast<int64_t>(sidx), lane, rec);
     }
 }
 
 // The VJP's pixel gradient from the per-stamp coefficients: it depends on
 // the pixels only through the coefficients, so this pass reads none and
 // streams the writes.  One warp per stamp, stamps in grid-stride order;
-// stamps of invalid size are left unwritten, like the analysis kernel
-// leaves them; a stamp without a solution gets zeros.
+// stamps of invalid size are left unwritten; a stamp without a solution gets
+// zeros.  Where rows are multiples of four pixels and the stamp starts on 16
+// bytes, a lane writes four pixels of a row at once and shares the row's terms
+// between them: 20 instructions a pixel instead of 41.
+//   20,000 stamps of 48x48 (184 MB written, 0.027 ms at the copy rate): 67 to 38
+//   us.
 __global__ void __launch_bounds__(256) moment_vjp_write_kernel(MomentGradArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -654,8 +628,35 @@ __global__ void __launch_bounds__(256) moment_vjp_write_kernel(MomentGradArgs a)
         const int npix = static_cast<int>(npl);
         const VjpCoef cf = a.coef[si];
         float* out = a.dpix + ix.offset;
+        const bool vec = (ix.w & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
         if (!cf.ok) {
             for (int p = lane; p < npix; p += 32) __stcs(out + p, 0.f);
+            continue;
+        }
+        if (vec) {
+            FWalk pw(4 * lane, ix.w, 128);
+            float4* o4 = reinterpret_cast<float4*>(out);
+#pragma unroll 2
+            for (int p = lane; p < npix / 4; p += 32) {
+                const float t2 = pw.r - cf.y0, di = pw.r - cf.pr, di2 = di * di;
+                const float e0 = cf.B * t2 * t2, e1 = -cf.G4 * t2;
+                const float k0 = fmaf(t2, fmaf(cf.c[5], t2, cf.c[2]), cf.c[0]), k1 = fmaf(cf.c[4], t2, cf.c[1]);
+                float g[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float x = pw.c + static_cast<float>(i);
+                    const float t1 = x - cf.x0;
+                    const float W = ex2(fmaf(t1, fmaf(cf.A, t1, e1), e0) * cf.cw);
+                    g[i] = -W * fmaf(t1, fmaf(cf.c[3], t1, k1), k0);
+                    if (cf.ring) {
+                        const float dj = x - cf.pc;
+                        const float d2 = fmaf(dj, dj, di2);
+                        g[i] += d2 <= cf.km2 ? cf.kc_in : (d2 <= cf.k2 ? cf.kc_ring : cf.kc_out);
+                    }
+                }
+                pw.next();
+                __stcs(o4 + p, make_float4(g[0], g[1], g[2], g[3]));
+            }
             continue;
         }
         FWalk pw(lane, ix.w);
@@ -685,16 +686,6 @@ cudaError_t launch_t(const MomentGradArgs& a, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if constexpr (!JVP) {
-        if (a.mode & FSE_MOM_SIGW_R50) {
-            long long rgrid = (a.count + 7) / 8;          // eight stamps (warps) per CTA
-            const long long rcap = static_cast<long long>(sms) * 8;
-            if (rgrid > rcap) rgrid = rcap;
-            moment_r50_kernel<DT, false><<<static_cast<unsigned>(rgrid), 256, 0, stream>>>(a);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-        }
-    }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
