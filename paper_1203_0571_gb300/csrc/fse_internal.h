@@ -94,6 +94,7 @@ struct GradArgs {
     float* dpix;             // laid out like pix (fp32), or NULL
     unsigned int* queue;     // work counter (zeroed before launch)
     const float2* bnf;       // the device's fp32 b(n), b'(n) table (bn_table_f32)
+    int aligned;             // pix, inv_var and dpix start on four-pixel boundaries (set at launch)
 };
 
 // Arguments of the star-profile kernel (fse_star_fit, Sec. 4.2).
