@@ -219,8 +219,10 @@ int fse_sersic_fit(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
 /* The whole chain of Sec. 4.1 (start-up, centroid + ellipticity from the
  * brightest pixel, fit) in three persistent launches on `stream`: the start-up
  * (brightest pixel, growth-curve r50, sigma_w), the moment iteration, then the
- * fit of every stamp whose moments converged.  Results are those of the three
- * single stages run in turn. */
+ * fit of every stamp whose moments converged.  A large batch (2048 warps'
+ * worth of stamps and more) runs as two such halves, the second on a stream of
+ * the context that `stream` waits for, unless `stream` is being captured.
+ * Results are those of the three single stages run in turn. */
 int fse_fit_batch(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
                   const fse_stamp *idx, int64_t count, const float *inv_var,
                   const fse_opts *opts, fse_result *out, void *stream);
@@ -238,8 +240,8 @@ int fse_fit_batch_plain(fse_ctx *ctx, const void *pix, int dtype, const float *s
  * the inputs to context-owned device buffers in chunks (from 8192 stamps up,
  * 9 chunks of 2, 4, 6, 8, 10, 10, 10, 8 and 6 64ths of the batch, else one)
  * on a context copy stream,
- * runs each chunk's chain on `stream` or a second context stream as soon as
- * its copy is done, copies the results back and returns when out[] is
+ * runs each chunk's chain on `stream` or one of five context streams as soon
+ * as its copy is done, copies the results back and returns when out[] is
  * complete.  npix_total bounds every idx[s].offset + h*w; a stamp outside it
  * returns FSE_EINVAL before any kernel runs, with out[] untouched (each chunk
  * is checked just before its copy, so the chunks before it may already have

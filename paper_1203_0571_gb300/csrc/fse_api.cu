@@ -34,6 +34,9 @@ constexpr int chunk_units_total() {
     return t;
 }
 static_assert(chunk_units_total() == 64, "the chunks must cover the batch in 64ths");
+constexpr int kHostStreams = 6;   // compute streams: the call's own and side streams
+
+constexpr int kSideStreams = fse::kClasses - 1;
 
 struct fse_ctx {
     int device = 0;
@@ -41,9 +44,8 @@ struct fse_ctx {
     unsigned int* d_queue = nullptr;   // kQueues slots of kQueueWords work counters
     unsigned int* d_err = nullptr;     // sticky error word written by the kernels
     unsigned next_queue = 0;
-    cudaStream_t aux_stream = nullptr; // second compute stream of the host-buffer pipeline
     cudaStream_t copy_stream = nullptr; // host-to-device copies of the host-buffer pipeline
-    cudaEvent_t chunk_ev[kHostChunks + 2] = {}; // chunk copies done; start; end
+    cudaEvent_t chunk_ev[kHostChunks + 1] = {}; // chunk copies done; the call's start
     // grow-only device staging of fse_fit_batch_host
     void* d_pix = nullptr;
     size_t pix_cap = 0;
@@ -60,11 +62,14 @@ struct fse_ctx {
     int32_t* d_perm = nullptr;
     size_t perm_cap = 0;
     unsigned int* d_cls = nullptr;
-    // one stream per size class but the largest, which runs on the call's own
-    // stream; fork: classification done; join[k]: class k done
-    cudaStream_t cls_stream[fse::kClasses - 1] = {};
-    cudaEvent_t cls_fork = nullptr;
-    cudaEvent_t cls_join[fse::kClasses - 1] = {};
+    // Streams for the parts of a call that run beside its own stream: the size
+    // classes of a ragged batch, the second half of a large one, the chunks of
+    // the host-buffer pipeline.  A part waits for `fork` (recorded on the call's
+    // stream), and the call's stream for `join` of every part.
+    cudaStream_t side[kSideStreams] = {};
+    cudaEvent_t fork = nullptr;
+    cudaEvent_t join[kSideStreams] = {};
+    unsigned next_side = 0;
     // grow-only per-stamp coefficients of fse_moment_vjp
     fse::VjpCoef* d_vjp = nullptr;
     size_t vjp_cap = 0;
@@ -81,7 +86,7 @@ struct fse_ctx {
 
 namespace {
 
-constexpr int kQueues = 64;                        // calls in flight on one context
+constexpr int kQueues = 128;                       // two for each call in flight on one context
 constexpr int kQueueWords = fse::kStageQueues;     // work counters of one call
 std::mutex g_table_mutex;
 // the context in which each device's b(n) table was built (0: not built); a
@@ -250,14 +255,58 @@ unsigned int* next_queue(fse_ctx* ctx) {
     return ctx->d_queue + static_cast<size_t>(ctx->next_queue++ % kQueues) * kQueueWords;
 }
 
-int run(fse_ctx* ctx, fse::LaunchArgs& a, cudaStream_t stream) {
+// Whether work of a call on `stream` may run beside it: not while the stream
+// is captured (the side streams would join the caller's capture).
+bool may_fork(cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone;
+}
+
+// One chain (or stage) on one stream.
+cudaError_t run_on(fse_ctx* ctx, const fse::LaunchArgs& a, cudaStream_t stream) {
+    fse::LaunchArgs b = a;
+    b.queue = next_queue(ctx);
+    const cudaError_t e = cudaMemsetAsync(b.queue, 0, kQueueWords * sizeof(unsigned int), stream);
+    return e != cudaSuccess ? e : fse::launch_estimator(b, stream);
+}
+
+// Warps a batch must bring for its second half to run beside the first: about
+// what the fit launch holds at once (16 warps on each of 152 SMs).
+constexpr int64_t kSplitWarps = 2048;
+
+// The whole chain of a large batch runs as two halves, the second on a side
+// stream: each of the chain's three launches ends in a tail of its slowest
+// stamps (0.45 ms a call on one stream, whatever its size), and the other
+// half's launches fill it.  Results do not depend on it.  100,000 stamps of
+// 48x48 5.86 to 5.68 ms, 20,000 1.54 to 1.39, 8,000 of 64x64 1.25 to 1.11, 3,000
+// of 48x48 0.51 to 0.50; three and four parts and uneven halves were no faster.
+int run(fse_ctx* ctx, const fse::LaunchArgs& a, cudaStream_t stream) {
     if (a.count == 0) return FSE_OK;
-    a.queue = next_queue(ctx);
-    cudaError_t e = cudaMemsetAsync(a.queue, 0, kQueueWords * sizeof(unsigned int), stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "work counter reset");
-    e = fse::launch_estimator(a, stream);
+    if (a.stage != fse::kStageAll || a.count * a.warps_per_stamp < kSplitWarps || !may_fork(stream)) {
+        const cudaError_t e = run_on(ctx, a, stream);
+        return e != cudaSuccess ? cuda_fail(ctx, e, "estimator launch") : FSE_OK;
+    }
+    const unsigned k = ctx->next_side++ % kSideStreams;
+    fse::LaunchArgs lo = a, hi = a;
+    lo.count = a.count / 2;
+    hi.count = a.count - lo.count;
+    hi.idx += lo.count;
+    hi.out += lo.count;
+    if (hi.scale) hi.scale += lo.count;
+    cudaError_t e = cudaEventRecord(ctx->fork, stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side[k], ctx->fork, 0);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "estimator launch");
-    return FSE_OK;
+    e = run_on(ctx, lo, stream);
+    if (e == cudaSuccess) e = run_on(ctx, hi, ctx->side[k]);
+    // join also after an error: the caller's buffers may be in use
+    cudaError_t j = cudaEventRecord(ctx->join[k], ctx->side[k]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(stream, ctx->join[k], 0);
+    if (e == cudaSuccess) e = j;
+    return e != cudaSuccess ? cuda_fail(ctx, e, "estimator launch") : FSE_OK;
 }
 
 int stage_entry(fse_ctx* ctx, const void* pix, int dtype, const float* scale, const fse_stamp* idx,
@@ -295,21 +344,6 @@ constexpr int kClsWords = (4 + kQueueWords) * kK;   // d_cls
 int ragged_workspace(fse_ctx* ctx, int64_t count) {
     int rc = grow(ctx, &ctx->d_perm, &ctx->perm_cap, static_cast<size_t>(count));
     if (rc) return rc;
-    if (!ctx->cls_fork) {
-        // first ragged call: the class streams and their events; kept on failure
-        // and completed by the next call
-        cudaError_t e = cudaSuccess;
-        for (int k = 0; k < kK - 1 && e == cudaSuccess; ++k) {
-            if (!ctx->cls_stream[k]) e = cudaStreamCreateWithFlags(&ctx->cls_stream[k], cudaStreamNonBlocking);
-            if (e == cudaSuccess && !ctx->cls_join[k])
-                e = cudaEventCreateWithFlags(&ctx->cls_join[k], cudaEventDisableTiming);
-        }
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->cls_fork, cudaEventDisableTiming);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return cuda_fail(ctx, e, "ragged streams");
-        }
-    }
     if (!ctx->d_cls) {
         cudaError_t e = cudaMalloc(&ctx->d_cls, kClsWords * sizeof(unsigned int));
         if (e != cudaSuccess) {
@@ -345,21 +379,23 @@ void class_shape(const fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o
 // tenth of its warps); one class after another pays 21 such tails in a row,
 // side by side one class's tail is filled by the others' stamps.
 // Event-ordered throughout, with no host synchronisation, so the sequence can
-// be captured.
-int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cudaStream_t s) {
+// be captured (into the context's own graph side by side; on a stream that the
+// caller captures, one class after another: fork = false).
+int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cudaStream_t s, bool fork) {
     unsigned int* counts = ctx->d_cls;
     unsigned int* range = counts + kK;
     unsigned int* cursor = range + 2 * kK;
     unsigned int* queues = cursor + kK;
     cudaError_t e = cudaMemsetAsync(ctx->d_cls, 0, kClsWords * sizeof(unsigned int), s);
     if (e == cudaSuccess) e = fse::classify_stamps(a.idx, a.count, counts, range, cursor, ctx->d_perm, s);
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->cls_fork, s);
+    if (e == cudaSuccess && fork) e = cudaEventRecord(ctx->fork, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "size classification");
     int forked = kK - 1;   // classes forked .. kK - 2 have work on their streams
     for (int k = kK - 1; k >= 0 && e == cudaSuccess; --k) {
-        const cudaStream_t ks = k == kK - 1 ? s : ctx->cls_stream[k];
-        if (k < kK - 1) {
-            e = cudaStreamWaitEvent(ks, ctx->cls_fork, 0);
+        cudaStream_t ks = s;
+        if (fork && k < kK - 1) {
+            ks = ctx->side[k];
+            e = cudaStreamWaitEvent(ks, ctx->fork, 0);
             if (e != cudaSuccess) break;
             forked = k;
         }
@@ -372,9 +408,9 @@ int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cu
         e = fse::launch_estimator(b, ks);
     }
     // join what was forked, also after an error: the caller's buffers are in use
-    for (int k = kK - 2; k >= forked; --k) {
-        cudaError_t j = cudaEventRecord(ctx->cls_join[k], ctx->cls_stream[k]);
-        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, ctx->cls_join[k], 0);
+    for (int k = kK - 2; fork && k >= forked; --k) {
+        cudaError_t j = cudaEventRecord(ctx->join[k], ctx->side[k]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, ctx->join[k], 0);
         if (e == cudaSuccess) e = j;
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "size-class launch");
@@ -470,20 +506,22 @@ int fse_create(fse_ctx** out, int device) {
         return FSE_ENOMEM;
     }
     if (cudaMemset(ctx->d_err, 0, sizeof(unsigned int)) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         fse_destroy(ctx);
         return FSE_ECUDA;
     }
-    for (cudaEvent_t& ev : ctx->chunk_ev) {
-        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-            ev = nullptr;
-            cudaGetLastError();
-            fse_destroy(ctx);
-            return FSE_ECUDA;
-        }
+    bool ok = cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int k = 0; k < kSideStreams && ok; ++k)
+        ok = cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&ctx->join[k], cudaEventDisableTiming) == cudaSuccess;
+    for (int k = 0; k < kHostChunks + 1 && ok; ++k)
+        ok = cudaEventCreateWithFlags(&ctx->chunk_ev[k], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        fse_destroy(ctx);
+        return FSE_ECUDA;
     }
     {
         std::lock_guard<std::mutex> lk(g_table_mutex);
@@ -512,13 +550,12 @@ void fse_destroy(fse_ctx* ctx) {
         cudaFree(ctx->d_perm);
         cudaFree(ctx->d_cls);
         cudaFree(ctx->d_vjp);
-        for (int k = 0; k < fse::kClasses - 1; ++k) {
-            if (ctx->cls_stream[k]) cudaStreamDestroy(ctx->cls_stream[k]);
-            if (ctx->cls_join[k]) cudaEventDestroy(ctx->cls_join[k]);
+        for (int k = 0; k < kSideStreams; ++k) {
+            if (ctx->side[k]) cudaStreamDestroy(ctx->side[k]);
+            if (ctx->join[k]) cudaEventDestroy(ctx->join[k]);
         }
-        if (ctx->cls_fork) cudaEventDestroy(ctx->cls_fork);
+        if (ctx->fork) cudaEventDestroy(ctx->fork);
         if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
-        if (ctx->aux_stream) cudaStreamDestroy(ctx->aux_stream);
         if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
         for (cudaEvent_t ev : ctx->chunk_ev)
@@ -618,17 +655,22 @@ int fse_fit_batch_host(fse_ctx* ctx, const void* pix, int64_t npix_total, int dt
         (scale && (rc = grow(ctx, &ctx->d_scale, &ctx->scale_cap, count))) ||
         (inv_var && (rc = grow(ctx, &ctx->d_ivar, &ctx->ivar_cap, npix_total))))
         return rc;
-    // Three streams: the copy stream moves every chunk's inputs to the device
-    // back to back and records chunk_ev[c] after chunk c; chunk c's kernels and
-    // its result copy run on compute stream c % 2 once chunk_ev[c] is done, so
-    // one chunk's launch tail overlaps the next chunk's kernels.
+    // The copy stream moves every chunk's inputs to the device back to back and
+    // records chunk_ev[c] after chunk c; chunk c's kernels and its result copy
+    // run on compute stream c % 6 once chunk_ev[c] is done.  A chunk's chain is
+    // at least as long as its slowest stamp's three launches (0.4 ms), so the
+    // chunks need several streams beside one another: with two, 40,000 stamps of
+    // 48x48 took 3.82 ms, three 3.37, four 3.22, six 3.18 (9,000 stamps 2.28,
+    // 1.68, 1.54, 1.29; 100,000 stamps 7.26, 7.00, 6.93, 6.93).
     const cudaStream_t s0 = static_cast<cudaStream_t>(stream);
-    const cudaStream_t streams[2] = {s0, ctx->aux_stream};
+    cudaStream_t streams[kHostStreams] = {s0};
+    for (int i = 1; i < kHostStreams; ++i) streams[i] = ctx->side[i - 1];
+    const int used = nchunk < kHostStreams ? nchunk : kHostStreams;
     const cudaStream_t cs = ctx->copy_stream;
-    cudaEvent_t ev_start = ctx->chunk_ev[kHostChunks], ev_end = ctx->chunk_ev[kHostChunks + 1];
+    cudaEvent_t ev_start = ctx->chunk_ev[kHostChunks];
     cudaError_t e = cudaEventRecord(ev_start, s0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ev_start, 0);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->aux_stream, ev_start, 0);
+    for (int i = 1; i < used && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(streams[i], ev_start, 0);
     // First, chunk by chunk: every stamp inside the pixel buffer, the largest
     // stamp, the chunk's pixel span [p_lo, p_hi), then the chunk's copies, so
     // that the first chunks move while the later ones are checked.  From
@@ -670,7 +712,7 @@ int fse_fit_batch_host(fse_ctx* ctx, const void* pix, int64_t npix_total, int dt
     for (int c = 0; c < nchunk && e == cudaSuccess; ++c) {
         const int64_t s_lo = lo[c], n_c = lo[c + 1] - lo[c];
         if (n_c == 0) continue;
-        const cudaStream_t st = streams[c & 1];
+        const cudaStream_t st = streams[c % kHostStreams];
         e = cudaStreamWaitEvent(st, ctx->chunk_ev[c], 0);
         if (e != cudaSuccess) break;
         fse::LaunchArgs a;
@@ -686,25 +728,18 @@ int fse_fit_batch_host(fse_ctx* ctx, const void* pix, int64_t npix_total, int dt
         a.opts = dev_opts(o);
         a.stage = fse::kStageAll;
         launch_shape(o, a.opts.max_pix, fse::kStageAll, &a.warps_per_cta, &a.warps_per_stamp);
-        rc = run(ctx, a, st);
-        if (rc) {
-            cudaStreamSynchronize(cs);
-            cudaStreamSynchronize(ctx->aux_stream);
-            cudaStreamSynchronize(s0);
-            cudaGetLastError();
-            return rc;
-        }
+        if ((e = run_on(ctx, a, st)) != cudaSuccess) break;
         e = cudaMemcpyAsync(out + s_lo, ctx->d_out + s_lo, n_c * sizeof(fse_result),
                             cudaMemcpyDeviceToHost, st);
     }
-    // the caller's stream waits for the other compute stream (whose work waited
-    // on the copy stream's events), then the call waits for the caller's stream
-    if (e == cudaSuccess) e = cudaEventRecord(ev_end, ctx->aux_stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, ev_end, 0);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s0);
+    // the call ends when every compute stream has (their work waited on the copy
+    // stream's events)
+    for (int i = 0; i < used; ++i) {
+        const cudaError_t j = cudaStreamSynchronize(streams[i]);
+        if (e == cudaSuccess) e = j;
+    }
     if (e != cudaSuccess) {
-        cudaStreamSynchronize(ctx->copy_stream);
-        cudaStreamSynchronize(ctx->aux_stream);
+        cudaStreamSynchronize(cs);
         return cuda_fail(ctx, e, "host-buffer pipeline");
     }
     unsigned int flag = 0;
@@ -730,7 +765,7 @@ int fse_fit_batch_ragged(fse_ctx* ctx, const void* pix, int dtype, const float* 
     if (rc || count == 0) return rc;
     if ((rc = ragged_workspace(ctx, count))) return rc;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (!(o.flags & FSE_FLAG_GRAPH)) return enqueue_ragged(ctx, a, o, s);
+    if (!(o.flags & FSE_FLAG_GRAPH)) return enqueue_ragged(ctx, a, o, s, may_fork(s));
     RaggedKey key;
     make_key(ctx, a, o, &key);
     if (!ctx->gexec || memcmp(&key, ctx->gkey, sizeof key) != 0) {
@@ -739,7 +774,7 @@ int fse_fit_batch_ragged(fse_ctx* ctx, const void* pix, int dtype, const float* 
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture");
-        rc = enqueue_ragged(ctx, a, o, ctx->cap_stream);
+        rc = enqueue_ragged(ctx, a, o, ctx->cap_stream, true);
         e = cudaStreamEndCapture(ctx->cap_stream, &graph);
         if (rc) {
             if (graph) cudaGraphDestroy(graph);
