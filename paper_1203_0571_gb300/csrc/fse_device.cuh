@@ -369,6 +369,13 @@ __device__ __forceinline__ Box weight_box(float xc, float yc, float g1, float g2
     return b;
 }
 
+// a / b for 0 <= a <= 256 and 1 <= b <= 128, from ib = 1 / b to a few ulps:
+// (a + 1/2) / b lies at least 1/256 from every integer, and the product is off
+// by less than 1e-4.
+__device__ __forceinline__ int div_small(int a, float ib) {
+    return static_cast<int>((static_cast<float>(a) + 0.5f) * ib);
+}
+
 // The pixels q = t, t + nt, ... of a box, row-major within it (the stamp
 // index p grows with q, so a walk ends once p passes the box's last pixel;
 // a thread with t beyond the box starts past it): their offsets
@@ -382,15 +389,16 @@ struct BoxWalk {
     float du, dv, wrap, fbw;
     int dp, dwrap;
     __device__ __forceinline__ BoxWalk(int t, const Box& b, int w, int nt, int xr, int yr) {
-        const int row = t / b.bw, col = t - row * b.bw;
-        const int dr = nt / b.bw, dc = nt - dr * b.bw;
+        fbw = static_cast<float>(b.bw);
+        const float ib = __fdividef(1.f, fbw);
+        const int row = div_small(t, ib), col = t - row * b.bw;
+        const int dr = div_small(nt, ib), dc = nt - dr * b.bw;
         u = static_cast<float>(b.c0 + col - xr);
         v = static_cast<float>(b.r0 + row - yr);
         p = (b.r0 + row) * w + b.c0 + col;
         du = static_cast<float>(dc);
         dv = static_cast<float>(dr);
         wrap = static_cast<float>(b.c0 + b.bw - xr);
-        fbw = static_cast<float>(b.bw);
         dp = dr * w + dc;
         dwrap = w - b.bw;
     }

@@ -304,6 +304,20 @@ struct Grp {
         return v;
     }
 
+    // Largest of a non-negative value over the group (as its bits, which order
+    // like the values; infinity above all).
+    __device__ __forceinline__ float max_nonneg(float v) const {
+        unsigned b = __reduce_max_sync(kFull, __float_as_uint(v));
+        if (NW > 1) {
+            sync();
+            if (lane == 0) red[wi * 32] = __uint_as_float(b);
+            sync();
+#pragma unroll
+            for (int k = 0; k < NW; ++k) b = max(b, __float_as_uint(red[k * 32]));
+        }
+        return __uint_as_float(b);
+    }
+
     __device__ __forceinline__ bool all(bool b) const {
         b = __all_sync(kFull, b);
         if (NW > 1) {
@@ -1636,7 +1650,7 @@ __device__ Precise refine_tail(const float (&rh)[10], const float (&rl)[10], con
 
 template <bool IVAR, int NW, bool SUP = false>
 __device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
-                              const float* __restrict__ sq, int w, int npix, const Grp<NW>& g,
+                              const float* __restrict__ sq, float qmax, int w, int npix, const Grp<NW>& g,
                               float I0g,
                               float re, float n, float lq, const MomState& st, int S = 1) {
     float bf, dbf;
@@ -1645,8 +1659,9 @@ __device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
     const float nbl = -bf * kLog2e;
     const float c0 = log2f(re) + lq;
     // fp64 model constants for the bright pixels of the final pass; a model
-    // value exceeds the threshold only if |I0| does (E <= 1)
-    const bool check_bright = IVAR || fabsf(I0g) > kBrightSigma;
+    // value (times sqrt(inv_var), at most qmax) exceeds the threshold only if
+    // |I0| does (E <= 1)
+    const bool check_bright = IVAR ? fabsf(I0g) * qmax > kBrightSigma : fabsf(I0g) > kBrightSigma;
     BrightModel bm;
     if (check_bright) {
         double dbd;
@@ -1809,7 +1824,7 @@ struct FitOut {
 // Levenberg-Marquardt over theta = (r_e, n) with I0 at its closed form after
 // every pass; damping by the gain ratio rho (Nielsen 1999).
 template <bool IVAR, int NW, bool SUP = false>
-__device__ FitOut sersic_fit(const float* s, uint32_t tm, const float* sq, int h, int w, int npix,
+__device__ FitOut sersic_fit(const float* s, uint32_t tm, const float* sq, float qmax, int h, int w, int npix,
                              const Grp<NW>& g, const DevOpts& o, const MomState& st,
                              uint32_t& status) {
     // per-pixel 0.5 log2 R^2 about the fixed centre with the fixed ellipticity
@@ -1821,14 +1836,15 @@ __device__ FitOut sersic_fit(const float* s, uint32_t tm, const float* sq, int h
     if constexpr (!SUP) {
         // eight columns of tensor memory at a time (the last ones may lie past
         // the stamp: values of no pixel, never read back)
-        PixelWalk pw(g.t, w, Grp<NW>::NT);
+        const Box whole = {0, 0, h, w};
+        BoxWalk pw(g.t, whole, w, Grp<NW>::NT, st.xi, st.yi);
 #pragma unroll 1
         for (int c = 0; c * Grp<NW>::NT < npix; c += 8) {
             float v[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const float t1 = static_cast<float>(pw.col - st.xi) - st.xf;
-                const float t2 = static_cast<float>(pw.row - st.yi) - st.yf;
+                const float t1 = pw.u - st.xf;
+                const float t2 = pw.v - st.yf;
                 const float R2 = fmaf(A, t1 * t1, fmaf(B, t2 * t2, -G4 * (t1 * t2)));
                 v[j] = half_log2_r2(R2);
                 pw.next();
@@ -1954,7 +1970,7 @@ __device__ FitOut sersic_fit(const float* s, uint32_t tm, const float* sq, int h
         int passes = 0;
 #pragma unroll 1
         for (;;) {
-            const Precise E = fit_refine<IVAR, NW, SUP>(s, tm, sq, w, npix, g, tI0, te, tn, lq, st, S);
+            const Precise E = fit_refine<IVAR, NW, SUP>(s, tm, sq, qmax, w, npix, g, tI0, te, tn, lq, st, S);
             ++passes;
             // a step within 1e-2 is taken on the Newton model alone: its chi^2
             // decrease can be below the rounding of the fp32 model values
@@ -2146,14 +2162,32 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 
             skip = true;
         }
         float* s = pixbuf;
+        float qmax = 0.f;
         if (!skip) {
             const char* gsrc = static_cast<const char*>(a.pix) + ix.offset * (DT == FSE_BF16 ? 2 : 4);
             const float scale = (DT == FSE_BF16 && a.scale) ? a.scale[si] : 1.f;
             const bool ok = stage_stamp<DT>(pixbuf, &s, aux, gsrc, static_cast<int>(npl), scale, bar,
                                             &phase, g);
             if (kIv && ok) {
+                // sqrt(inv_var), eight loads in flight per thread, and its largest
                 const float* gv = a.inv_var + ix.offset;
-                for (int p = g.t; p < npl; p += Grp<NW>::NT) ivbuf[p] = sqrtf(fmaxf(__ldg(gv + p), 0.f));
+#pragma unroll 1
+                for (int p0 = g.t; p0 < npl; p0 += 8 * Grp<NW>::NT) {
+                    float v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int p = p0 + u * Grp<NW>::NT;
+                        v[u] = p < npl ? __ldg(gv + p) : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int p = p0 + u * Grp<NW>::NT;
+                        const float q = sqrtf(fmaxf(v[u], 0.f));
+                        qmax = fmaxf(qmax, q);
+                        if (p < npl) ivbuf[p] = q;
+                    }
+                }
+                qmax = g.max_nonneg(qmax);
                 g.sync();
             }
             if (!ok) {
@@ -2253,7 +2287,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 
             }
         }
         if (!skip && (STAGE == kStageFit || STAGE == kStageAll)) {
-            const FitOut f = sersic_fit<IVAR, NW, SUP>(s, tm, ivbuf, h, w, npix, g, o, st, status);
+            const FitOut f = sersic_fit<IVAR, NW, SUP>(s, tm, ivbuf, qmax, h, w, npix, g, o, st, status);
             res.I0 = static_cast<float>(f.I0);
             res.re = static_cast<float>(f.re);
             res.n = static_cast<float>(f.n);
