@@ -615,9 +615,11 @@ __device__ __forceinline__ void moment_pass(const float* __restrict__ s, int w, 
     const float cy = static_cast<float>(st.yi - st.yr) + st.yf;
     // pixel offsets from the reference pixel, exact integers in fp32
     BoxWalk ow(g.t, bx, w, Grp<NW>::NT, st.xr, st.yr);
-    const int plast = bx.last(w);   // the walk's index grows with each step
+    const int area = bx.bh * bx.bw;
+    // (a count of steps: comparing the walk's index with the box's last pixel
+    // put the exit of every step behind the walk; 7 % of the moment launch)
 #pragma unroll 2
-    while (ow.p <= plast) {
+    for (int left = area - g.t; left > 0; left -= Grp<NW>::NT) {
         const float t1 = ow.u - cx;
         const float t2 = ow.v - cy;
         const float I = s[ow.p];
@@ -834,9 +836,9 @@ __device__ float moment_refine(const float* __restrict__ s, int h, int w, const 
     for (int i = 0; i < 6; ++i) dh[i] = dl[i] = cx[i] = 0.f;
     const Box bx = weight_box(st, h, w);
     BoxWalk ow(g.t, bx, w, Grp<NW>::NT, st.xi, st.yi);
-    const int plast = bx.last(w);
+    const int area = bx.bh * bx.bw;
 #pragma unroll 1
-    while (ow.p <= plast) {
+    for (int left = area - g.t; left > 0; left -= Grp<NW>::NT) {
         const int p = ow.p;
         const float k1 = ow.u, k2 = ow.v;
         // theta = k - x_f exactly as hi + lo (|k| >= |x_f| unless k = 0, where lo = 0)
