@@ -19,6 +19,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "fse_device.cuh"
 #include "fse_internal.h"
@@ -1558,6 +1559,22 @@ __device__ __noinline__ double bright_r2(const BrightModel& bm, double t1, doubl
     return r * r;
 }
 
+// The constants of bright_r2 (out of line as well: few stamps need them).
+__device__ __noinline__ BrightModel bright_model(const MomState& st, float re, float n, float I0g) {
+    BrightModel bm;
+    double dbd;
+    bn_eval(static_cast<double>(n), &bm.b, &dbd);
+    bm.lnre = log(static_cast<double>(re));
+    const double g1 = st.g1, g2 = st.g2, gg = g1 * g1 + g2 * g2;
+    bm.ln1g = log(1.0 - sqrt(gg));
+    bm.A = 1.0 + gg - 2.0 * g1;
+    bm.B = 1.0 + gg + 2.0 * g1;
+    bm.G4 = 4.0 * g2;
+    bm.inv_n = 1.0 / static_cast<double>(n);
+    bm.I0 = I0g;
+    return bm;
+}
+
 // The same for the pixel-integrated model: the mean over the S x S sub-grid.
 __device__ __noinline__ double bright_r2_sub(const BrightModel& bm, double t1, double t2, float pix,
                                              float q, int S) {
@@ -1665,26 +1682,15 @@ __device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
     // |I0| does (E <= 1)
     const bool check_bright = IVAR ? fabsf(I0g) * qmax > kBrightSigma : fabsf(I0g) > kBrightSigma;
     BrightModel bm;
-    if (check_bright) {
-        double dbd;
-        bn_eval(static_cast<double>(n), &bm.b, &dbd);
-        bm.lnre = log(static_cast<double>(re));
-        const double g1 = st.g1, g2 = st.g2, gg = g1 * g1 + g2 * g2;
-        bm.ln1g = log(1.0 - sqrt(gg));
-        bm.A = 1.0 + gg - 2.0 * g1;
-        bm.B = 1.0 + gg + 2.0 * g1;
-        bm.G4 = 4.0 * g2;
-        bm.inv_n = 1.0 / static_cast<double>(n);
-        bm.I0 = I0g;
-    }
+    if (check_bright) bm = bright_model(st, re, n, I0g);
     float rh[10], rl[10], T[4];
 #pragma unroll
     for (int i = 0; i < 10; ++i) rh[i] = rl[i] = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) T[i] = 0.f;
-    PixelWalk pw(g.t, w, Grp<NW>::NT);
     if constexpr (SUP) {
         // the pixel-integrated model: every factor below is a mean over the sub-grid
+        PixelWalk pw(g.t, w, Grp<NW>::NT);
         const SubGeom sg = sub_geom(st, S);
         for (int p = g.t; p < npix; p += Grp<NW>::NT) {
             float t1, t2;
@@ -1754,22 +1760,25 @@ __device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
             }
         }
     } else {
-        tm_pixels<1, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) {
+        // one pixel; kBright: tested against the threshold (a loop of its own, so
+        // that the usual one holds only its own code)
+        auto pixel = [&](int p, float a, auto tested) {
+            constexpr bool kBright = decltype(tested)::value;
             const float u = exp2_acc(a * inv_n);
             float E = exp2_acc<true>(u * nbl);
             float r = fmaf(I0g, E, -s[p]);
             float rr_hi = 0.f, rr_lo = 0.f;
             bool bright = false;
-            if (check_bright) {
+            if constexpr (kBright) {
                 const float q = IVAR ? sq[p] : 1.f;
                 if (fabsf(I0g * E) * q > kBrightSigma) {
-                    const double rrd = bright_r2(bm, static_cast<double>(pw.col - st.xi) - st.xf,
-                                                 static_cast<double>(pw.row - st.yi) - st.yf, s[p], q);
+                    const int row = p / w, col = p - row * w;
+                    const double rrd = bright_r2(bm, static_cast<double>(col - st.xi) - st.xf,
+                                                 static_cast<double>(row - st.yi) - st.yf, s[p], q);
                     rr_hi = static_cast<float>(rrd);
                     rr_lo = static_cast<float>(rrd - rr_hi);
                     bright = true;
                 }
-                pw.next();
             }
             if (IVAR) {
                 const float q = sq[p];
@@ -1795,13 +1804,17 @@ __device__ Precise fit_refine(const float* __restrict__ s, uint32_t tm,
             T[1] = fmaf(vr, u, T[1]);        // r E u^2
             T[2] = fmaf(var, u, T[2]);       // r E u^2 a
             T[3] = fmaf(var * u, a, T[3]);   // r E u^2 a^2
-            if (bright) {
+            if (kBright && bright) {
                 df_add(rh[9], rl[9], rr_hi);
                 rl[9] += rr_lo;
             } else {
                 df_add(rh[9], rl[9], r * r);
             }
-        });
+        };
+        if (check_bright)
+            tm_pixels<1, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) { pixel(p, a, std::true_type{}); });
+        else
+            tm_pixels<1, Grp<NW>::NT>(tm, g.t, npix, c0, [&](int p, float a) { pixel(p, a, std::false_type{}); });
     }
     g.allsum_df(rh, rl);
     g.allsum(T);
