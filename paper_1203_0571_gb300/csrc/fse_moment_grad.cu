@@ -633,45 +633,45 @@ __global__ void __launch_bounds__(256) moment_vjp_write_kernel(MomentGradArgs a)
             for (int p = lane; p < npix; p += 32) __stcs(out + p, 0.f);
             continue;
         }
+        // one value from a row's terms and a column: the same operations on both
+        // paths, so that a gradient does not depend on where its stamp starts
+        float t2, di2, e0, e1, k0, k1;
+        auto row = [&](float r) {
+            t2 = r - cf.y0;
+            const float di = r - cf.pr;
+            di2 = di * di;
+            e0 = cf.B * t2 * t2;
+            e1 = -cf.G4 * t2;
+            k0 = fmaf(t2, fmaf(cf.c[5], t2, cf.c[2]), cf.c[0]);
+            k1 = fmaf(cf.c[4], t2, cf.c[1]);
+        };
+        auto value = [&](float x) {
+            const float t1 = x - cf.x0;
+            const float W = ex2(fmaf(t1, fmaf(cf.A, t1, e1), e0) * cf.cw);
+            float g = -W * fmaf(t1, fmaf(cf.c[3], t1, k1), k0);
+            if (cf.ring) {
+                const float dj = x - cf.pc;
+                const float d2 = fmaf(dj, dj, di2);
+                g += d2 <= cf.km2 ? cf.kc_in : (d2 <= cf.k2 ? cf.kc_ring : cf.kc_out);
+            }
+            return g;
+        };
         if (vec) {
             FWalk pw(4 * lane, ix.w, 128);
             float4* o4 = reinterpret_cast<float4*>(out);
 #pragma unroll 2
             for (int p = lane; p < npix / 4; p += 32) {
-                const float t2 = pw.r - cf.y0, di = pw.r - cf.pr, di2 = di * di;
-                const float e0 = cf.B * t2 * t2, e1 = -cf.G4 * t2;
-                const float k0 = fmaf(t2, fmaf(cf.c[5], t2, cf.c[2]), cf.c[0]), k1 = fmaf(cf.c[4], t2, cf.c[1]);
-                float g[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float x = pw.c + static_cast<float>(i);
-                    const float t1 = x - cf.x0;
-                    const float W = ex2(fmaf(t1, fmaf(cf.A, t1, e1), e0) * cf.cw);
-                    g[i] = -W * fmaf(t1, fmaf(cf.c[3], t1, k1), k0);
-                    if (cf.ring) {
-                        const float dj = x - cf.pc;
-                        const float d2 = fmaf(dj, dj, di2);
-                        g[i] += d2 <= cf.km2 ? cf.kc_in : (d2 <= cf.k2 ? cf.kc_ring : cf.kc_out);
-                    }
-                }
+                row(pw.r);
+                const float4 g = make_float4(value(pw.c), value(pw.c + 1.f), value(pw.c + 2.f), value(pw.c + 3.f));
                 pw.next();
-                __stcs(o4 + p, make_float4(g[0], g[1], g[2], g[3]));
+                __stcs(o4 + p, g);
             }
             continue;
         }
         FWalk pw(lane, ix.w);
         for (int p = lane; p < npix; p += 32) {
-            const float t1 = pw.c - cf.x0, t2 = pw.r - cf.y0;
-            const float R2 = fmaf(cf.A, t1 * t1, fmaf(cf.B, t2 * t2, -cf.G4 * (t1 * t2)));
-            const float W = ex2(R2 * cf.cw);
-            const float Q = fmaf(t1, fmaf(cf.c[3], t1, fmaf(cf.c[4], t2, cf.c[1])),
-                                 fmaf(t2, fmaf(cf.c[5], t2, cf.c[2]), cf.c[0]));
-            float g = -W * Q;
-            if (cf.ring) {
-                const float dj = pw.c - cf.pc, di = pw.r - cf.pr;
-                const float d2 = fmaf(di, di, dj * dj);
-                g += d2 <= cf.km2 ? cf.kc_in : (d2 <= cf.k2 ? cf.kc_ring : cf.kc_out);
-            }
+            row(pw.r);
+            const float g = value(pw.c);
             pw.next();
             __stcs(out + p, g);
         }
