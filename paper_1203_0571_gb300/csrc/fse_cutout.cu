@@ -134,8 +134,8 @@ __device__ __forceinline__ float max_abs_nan(float a, float b) {
 constexpr int kNear = 24;                 // half-side of the square, and its last ring
 constexpr int kFixBits = 22;              // piece width of the total and the near rings (at
                                           // most 200 pixels each)
-constexpr int kBlock = 128;               // vectors a thread sums before it empties its pieces
-                                          // (at most 2^10 pixels)
+constexpr int kBlock = 127;               // vectors a thread sums before it empties its pieces
+                                          // (fewer than 2^10 pixels of |q0| <= 2^21)
 constexpr int kFarBits = 17;              // piece width of the whole image's rings (at most
                                           // 2^14 pixels each)
 constexpr int kRun = 4;                   // consecutive pixels a thread bins at a time (2: 0.242
@@ -342,8 +342,8 @@ __global__ void __cluster_dims__(kCutCluster, 1, 1) __launch_bounds__(kCutThread
             const bool two = npix >= (1 << 18) && !fx.wide;   // |q| < 2^44: two pieces do
             for (int j0 = tid; j0 < rg.nvec; j0 += kBlock * kCutThreads) {
                 const int jend = min(rg.nvec, j0 + kBlock * kCutThreads);
-                const int n = (jend - j0 + kCutThreads - 1) / kCutThreads * N;
-                int t0 = 0, t1 = 0, t2 = 0;
+                const unsigned n = (jend - j0 + kCutThreads - 1) / kCutThreads * N;
+                unsigned t0 = 0, t1 = 0, t2 = 0;   // modulo 2^32: only the difference is small
                 if (two) {
 #pragma unroll 4
                     for (int j = j0; j < jend; j += kCutThreads) {
@@ -384,7 +384,8 @@ __global__ void __cluster_dims__(kCutCluster, 1, 1) __launch_bounds__(kCutThread
                         }
                     }
                 }
-                tot += fix_join(fx, t0 - n * kFixBias, t1 - n * kFixBias, t2 - n * kFixBias);
+                tot += fix_join(fx, static_cast<int>(t0 - n * kFixBias), static_cast<int>(t1 - n * kFixBias),
+                                static_cast<int>(t2 - n * kFixBias));
             }
             const int r0 = max(0, pr - kNear), r1 = min(ix.h - 1, pr + kNear);
             const int c0 = max(0, pc - kNear), c1 = min(ix.w - 1, pc + kNear);

@@ -1167,7 +1167,7 @@ __device__ InitOut stamp_init(const float* s, int h, int w, int npix, const Grp<
     }
     long long tot;
     {
-        int t0 = 0, t1 = 0, t2 = 0, n = 0;
+        unsigned t0 = 0, t1 = 0, t2 = 0, n = 0;   // modulo 2^32: only the difference is small
         if (!fx.wide) {
 #pragma unroll 4
             for (int p = g.t; p < npix; p += NT) {
@@ -1189,7 +1189,8 @@ __device__ InitOut stamp_init(const float* s, int h, int w, int npix, const Grp<
                 ++n;
             }
         }
-        tot = g.allsum_ll(fix_join(fx, t0 - n * kFixBias, t1 - n * kFixBias, t2 - n * kFixBias));
+        tot = g.allsum_ll(fix_join(fx, static_cast<int>(t0 - n * kFixBias), static_cast<int>(t1 - n * kFixBias),
+                                   static_cast<int>(t2 - n * kFixBias)));
     }
     if (tot <= 0) {
         o.fallback = true;
