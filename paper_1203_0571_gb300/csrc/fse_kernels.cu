@@ -3,15 +3,16 @@
 // with an elliptical weight (Sec. 3, Appendices A and B) and the Sérsic
 // profile fit with I0 at its closed form (Sec. 4.1, Eqs. 10-13).
 //
-// Execution model: two persistent launches per batch (the start-up and moment
-// iteration, then the fit); in each, every warp owns one stamp at a time
-// and takes the next from an atomic work counter.  The stamp is staged once
-// HBM -> shared memory (1-D TMA bulk copy for its 16-byte-aligned body, plain
-// loads for the ragged ends) and every later pass (start-up, moment
-// iterations, fit iterations) reads shared memory only.  Per pixel the work is
-// fp32 (MUFU ex2 for the weight and the profile); per-lane partial sums are
-// reduced with xor shuffles, which give every lane the same total, so all
-// lanes run the scalar update redundantly and stay in lock-step.
+// Execution model: three persistent launches per batch (start-up, moment
+// iteration, fit); in each, every warp (or group of NW warps, for large
+// stamps) owns one stamp at a time and takes the next from an atomic work
+// counter.  The stamp is staged once HBM -> shared memory (1-D TMA bulk copy
+// for its 16-byte-aligned body, plain loads for the ragged ends) and every
+// later pass reads shared memory only; the fit keeps each pixel's log radius
+// in tensor memory.  Per pixel the work is fp32 (MUFU ex2 for the weight and
+// the profile); per-lane partial sums are exchanged until every lane holds the
+// same totals, so all lanes run the scalar update redundantly and stay in
+// lock-step.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
