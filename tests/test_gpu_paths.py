@@ -11,6 +11,7 @@ from paper_1203_0571_gb300 import binding as B
 from paper_1203_0571_gb300 import synth
 from test_gpu_adjoint import check_against_oracle as check_adjoint
 from test_gpu_cutout import check_against_oracle as check_cutout
+from test_gpu_star import compare as compare_stars, gpu_stars, oracle_moments, oracle_stars
 
 pytestmark = pytest.mark.gpu
 
@@ -176,3 +177,21 @@ def test_cutout_passes(ctx, O, lead, dtype):
     torch.cuda.synchronize()
     inf = check_cutout(O, batch, out, cidx, info)
     assert np.any(inf["r50"] < 20) and np.any(inf["r50"] > 30)
+
+
+@pytest.mark.parametrize("h,w", [(15, 15), (16, 16), (16, 17), (17, 21), (22, 16), (25, 25), (23, 32), (32, 32)])
+def test_star_window_remainders(ctx, O, h, w):
+    """Pixel counts whose last step of 256 holds none, a few, up to three and
+    more pixels per lane, with and without lanes that have all eight, in the
+    Gaussian weight's loop: the star file's own comparison with the oracle."""
+    rng = np.random.default_rng(h * w)
+    stamps = [synth.single_stamp(h, w, n=0.5, re=float(rng.uniform(1.6, 2.4)), g1=float(rng.uniform(-0.1, 0.1)),
+                                 g2=float(rng.uniform(-0.1, 0.1)), xc=w / 2 - 0.5 + float(rng.uniform(-0.4, 0.4)),
+                                 yc=h / 2 - 0.5 + float(rng.uniform(-0.4, 0.4)), I0=1500.0, noise_sigma=1.0,
+                                 seed=int(rng.integers(1 << 30))) for _ in range(8)]
+    batch = synth.StampBatch(pix=torch.as_tensor(np.concatenate([s.astype(np.float32).ravel() for s in stamps])),
+                             offset=torch.arange(8) * h * w, h=torch.full((8,), h, dtype=torch.int32),
+                             w=torch.full((8,), w, dtype=torch.int32), truth={})
+    mom = oracle_moments(O, batch)
+    compare_stars(gpu_stars(ctx, batch, mom, "gauss"), oracle_stars(O, batch, mom, "gauss"), mom, "gauss",
+                  min_converged=0.5)
