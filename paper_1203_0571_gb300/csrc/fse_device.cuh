@@ -414,6 +414,18 @@ struct BoxWalk {
     }
 };
 
+// The first candidate of the growth curve's crossing ring from a recorded r50 =
+// (k - 1) + frac, frac in (0, 1].  The record is the caller's, so a radius past
+// the stamp (infinity included) stops at the ring h + w + 8: every pixel lies
+// within h + w, so the search's eight steps end without a crossing, as they do
+// from any farther ring, and neither the ring's box nor k^2 can leave 32 bits.
+// NaN and radii up to 1/2 start at the brightest pixel.
+__host__ __device__ inline int ring_guess(float r50, int h, int w) {
+    const int far = h + w + 8;
+    if (!(r50 > 0.5f)) return 0;
+    return r50 < static_cast<float>(far) ? static_cast<int>(ceilf(r50)) : far;
+}
+
 // b(n), b'(n) in fp32 from a table of (b, b') at n = kBnLo + k kBnStep:
 // cubic Hermite interpolation for b; b' as the linear interpolation of the
 // node values of b' (error O(h^2 b''') ~ 1e-9).  Differentiating the

@@ -239,8 +239,7 @@ __device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, float 
     o.c_in = o.c_ring = o.c_out = o.u_in = o.u_disc = 0.f;
     const float tot = tot_h + tot_l;
     if (!(tot > 0.f)) return o;                  // fallback radius: no dependence
-    // candidate from the start-up radius: r50 = (k-1) + frac, frac in (0, 1]
-    int k = r50_hint > 0.5f ? static_cast<int>(ceilf(r50_hint)) : 0;
+    int k = ring_guess(r50_hint, ix.h, ix.w);   // candidate from the start-up radius
 #pragma unroll 1
     for (int tries = 0; tries < 8; ++tries) {
         float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
