@@ -113,18 +113,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // moves K registers per lane (.32x32b.xK).  Warp w of a CTA reaches the 32
 // lanes of quadrant w % 4 only.  The loads are asynchronous: their registers
 // are ready after the wait, which takes them as operands so that no use moves
-// above it.
+// above it.  Every one of these instructions wants the whole warp at once
+// (.sync.aligned), whatever branches the code before it took: each function
+// first brings the warp together.
 __device__ __forceinline__ void tm_store8(uint32_t addr, const float (&v)[8]) {
+    __syncwarp();
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr),
                  "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
                  : "memory");
 }
 
 __device__ __forceinline__ void tm_wait_store() {
+    __syncwarp();
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[1]) {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
                  : "=f"(v[0])
                  : "r"(addr)
@@ -132,10 +137,12 @@ __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[1]) {
 }
 
 __device__ __forceinline__ void tm_wait(float (&v)[1]) {
+    __syncwarp();
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]) : : "memory");
 }
 
 __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[2]) {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
                  : "=f"(v[0]), "=f"(v[1])
                  : "r"(addr)
@@ -143,10 +150,12 @@ __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[2]) {
 }
 
 __device__ __forceinline__ void tm_wait(float (&v)[2]) {
+    __syncwarp();
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]) : : "memory");
 }
 
 __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[4]) {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
                  : "r"(addr)
@@ -154,10 +163,12 @@ __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[4]) {
 }
 
 __device__ __forceinline__ void tm_wait(float (&v)[4]) {
+    __syncwarp();
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]) : : "memory");
 }
 
 __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[8]) {
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "r"(addr)
@@ -165,10 +176,24 @@ __device__ __forceinline__ void tm_load(uint32_t addr, float (&v)[8]) {
 }
 
 __device__ __forceinline__ void tm_wait(float (&v)[8]) {
+    __syncwarp();
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
                  :
                  : "memory");
+}
+
+// Columns for the CTA, by one warp: their address to *base; and their release.
+__device__ __forceinline__ void tm_alloc(uint32_t* base, int columns) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(base)), "r"(columns)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tm_free(uint32_t base, int columns) {
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(columns) : "memory");
 }
 
 // Calls body(p, a) for the thread's pixels p = t, t + NT, ... in order, with
@@ -183,7 +208,6 @@ __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0
     int c = 0;
     if (full >= K) {
         float v[K], a[K];
-        __syncwarp();
         tm_load(tm, v);
         tm_wait(v);
 #pragma unroll
@@ -191,7 +215,6 @@ __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0
 #pragma unroll 1
         for (; c + K <= full; c += K) {
             const int next = c + 2 * K <= full ? c + K : c;   // (the last load is not used)
-            __syncwarp();
             tm_load(tm + next, v);
 #pragma unroll
             for (int j = 0; j < K; ++j) body(t + NT * (c + j), a[j]);
@@ -204,7 +227,6 @@ __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0
 #pragma unroll 1
         for (; c + 2 <= full; c += 2) {
             float v[2];
-            __syncwarp();
             tm_load(tm + c, v);
             tm_wait(v);
 #pragma unroll
@@ -214,7 +236,6 @@ __device__ __forceinline__ void tm_pixels(uint32_t tm, int t, int npix, float c0
 #pragma unroll 1
     for (; c * NT < npix; ++c) {
         float v[1];
-        __syncwarp();
         tm_load(tm + c, v);
         tm_wait(v);
         if (t + NT * c < npix) body(t + NT * c, v[0] - c0);
@@ -2095,12 +2116,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 
     __shared__ uint32_t tm_base;
     uint32_t tm = 0;
     if constexpr (kTm) {
-        if (warp == 0) {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tm_base)),
-                         "r"(a.tm_alloc)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        if (warp == 0) tm_alloc(&tm_base, a.tm_alloc);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -2321,9 +2337,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (warp == 0)
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm_base), "r"(a.tm_alloc)
-                         : "memory");
+        if (warp == 0) tm_free(tm_base, a.tm_alloc);
     }
 }
 

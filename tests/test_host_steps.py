@@ -1,6 +1,8 @@
 """Index and rounding steps that the kernels take from fse_device.cuh, compiled
 for the host from that header and run on the CPU."""
 import ctypes
+import os
+import re
 import subprocess
 
 import pytest
@@ -50,3 +52,21 @@ def test_ring_candidate_stays_in_range(steps, h, w):
                 bh, bw = min(h - 1, pr + kk) - r0 + 1, min(w - 1, pc + kk) - c0 + 1
                 assert 1 <= bh <= h - r0 and 1 <= bw <= w - c0
                 assert 0 <= (r0 + bh - 1) * w + c0 + bw - 1 < h * w
+
+
+def test_warp_wide_instructions_meet_a_whole_warp():
+    """Every tensor-memory instruction that a whole warp has to execute together
+    (.sync.aligned) stands in a function that begins by bringing the warp
+    together: its callers branch per lane."""
+    for src in _build.SOURCES:
+        with open(os.path.join(_build.CSRC, src)) as f:
+            body, found = [], 0
+            for line in f:
+                if re.match(r"(template|__device__|__global__|\}|struct )", line):
+                    body = []
+                body.append(line.strip())
+                if re.search(r'"tcgen05\.[^"]*\.sync\.aligned', line):
+                    found += 1
+                    assert body[0].startswith("__device__ __forceinline__ void tm_"), (src, line)
+                    assert body[1] == "__syncwarp();", (src, body[0])
+            assert src != "fse_kernels.cu" or found >= 5
