@@ -134,8 +134,9 @@ __device__ __forceinline__ float max_abs_nan(float a, float b) {
 constexpr int kNear = 24;                 // half-side of the square, and its last ring
 constexpr int kFixBits = 22;              // piece width of the total and the near rings (at
                                           // most 200 pixels each)
-constexpr int kBlock = 127;               // vectors a thread sums before it empties its pieces
-                                          // (fewer than 2^10 pixels of |q0| <= 2^21)
+constexpr int kBlock = 127;               // vectors a thread sums before it empties its pieces:
+                                          // fewer than 2^10 pixels of |q0| <= 2^21 (and, of two
+                                          // pieces, npix / 2^11 pixels of |q1| <= 2^40 / npix)
 constexpr int kFarBits = 17;              // piece width of the whole image's rings (at most
                                           // 2^14 pixels each)
 constexpr int kRun = 4;                   // consecutive pixels a thread bins at a time (2: 0.242
@@ -358,18 +359,20 @@ __global__ void __cluster_dims__(kCutCluster, 1, 1) __launch_bounds__(kCutThread
                     }
                     t2 = n * kFixBias;
                 } else if (fx.wide) {
+                    // 64-bit values one by one, modulo 2^64 (their pieces run to
+                    // 2^22, not to half of it either way, and a block of bf16
+                    // vectors has too many of those for 32 bits)
+                    unsigned long long t = 0;
 #pragma unroll 1
                     for (int j = j0; j < jend; j += kCutThreads) {
                         float v[N];
                         ImgVec<DT>::get(__ldg(rg.body + j), sc, v);
 #pragma unroll 1
-                        for (int i = 0; i < N; ++i) {
-                            fix_split(fx, v[i], q0, q1, q2);
-                            t0 += q0;
-                            t1 += q1;
-                            t2 += q2;
-                        }
+                        for (int i = 0; i < N; ++i)
+                            t += static_cast<unsigned long long>(__float2ll_rn(v[i] * fx.up0));
                     }
+                    tot = static_cast<long long>(static_cast<unsigned long long>(tot) + t);
+                    continue;
                 } else {
 #pragma unroll 2
                     for (int j = j0; j < jend; j += kCutThreads) {

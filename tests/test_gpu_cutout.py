@@ -203,3 +203,28 @@ def test_cutout_edge_cases(ctx):
         with pytest.raises(B.FseError):
             ctx.cutout(batch.pix, idx, out=small, **kw)
     ctx.cutout(batch.pix, idx[:0], out=small)
+
+
+def test_cutout_total_of_saturated_values(ctx):
+    """Finite pixels whose largest value times their number overflows fp32: the
+    fixed-point values saturate at 64 bits and the sums wrap, the same for bf16
+    images (1,016 pixels of a thread between two emptyings of its 32-bit sums)
+    as for the fp32 images of the same values (508).  Two saturated pixels
+    cancel to -1 next to the centre; the others are 2^24 - 2^22 - 1 each, whose
+    lowest piece is as large as it can be, so half the light lies within
+    sqrt(area / 2 pi)."""
+    side, s = 1100, float(np.float32(0xBFFFFF * 2.0 ** -23))
+    img = torch.full((side, side), 2.0 ** -39, dtype=torch.float32)
+    img[550, 550] = 2.0 ** 110
+    img[550, 552] = -2.0 ** 110
+    bf = img.to(torch.bfloat16).cuda().ravel()
+    assert torch.equal(bf.float().cpu(), img.ravel())
+    idx = B.make_index(torch.zeros(1, dtype=torch.int64), torch.full((1,), side, dtype=torch.int32),
+                       torch.full((1,), side, dtype=torch.int32))
+    res = []
+    for pix, scale in ((bf, torch.tensor([s], device="cuda")), (bf.float() * s, None)):
+        _, _, info = ctx.cutout(pix, idx, scale=scale)
+        res.append(info.cpu())
+    assert torch.equal(res[0], res[1]), [r.view(torch.float32)[0, 4] for r in res]
+    r50 = float(res[0].view(torch.float32)[0, 4])
+    assert abs(r50 - (side * side / (2 * np.pi)) ** 0.5) < 1.0, r50
