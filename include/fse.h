@@ -420,8 +420,13 @@ int fse_sersic_b(fse_ctx *ctx, const double *n, double *b, double *db, int64_t c
  * respect to the centre or the ellipticity, and d|g|/dg is taken as 0 at
  * g = 0.  A stamp whose size is outside [1, FSE_MAX_PIX], or whose parameters
  * are not finite or lie outside r_e > 0, |g| < 1, n in [0.129, 10.27] (the
- * b(n) table), gets NaN in chi2, dparams and (for a valid size) dpix.  All
- * arrays are device pointers; asynchronous on `stream`. */
+ * b(n) table), gets NaN in chi2, dparams and (for a valid size) dpix.  The bits
+ * of chi2 and dpix depend neither on where a stamp starts in the buffers nor on
+ * the outputs asked for.  dparams is summed in one of two orders: for a width
+ * that is a multiple of four it rounds differently (about 1e-7 of its terms'
+ * sum) for a stamp that starts on a multiple of four elements of 16-byte aligned
+ * buffers (bf16: 8) than for one that does not, and with inv_var than with
+ * inv_var and dpix.  All arrays are device pointers; asynchronous on `stream`. */
 int fse_sersic_chi2_grad(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
                          const fse_stamp *idx, int64_t count, const float *inv_var,
                          const float *params, const double *gout, double *chi2,

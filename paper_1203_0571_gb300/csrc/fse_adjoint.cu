@@ -43,7 +43,13 @@ namespace {
 // about half the instructions per pixel of the lane-strided form.  The
 // arithmetic of a pixel is the same in both; chi^2 is summed in the strided
 // form's order in both (a warp's squared residuals pass through shared memory),
-// so its bits depend neither on the form nor on the outputs asked for.
+// so its bits depend neither on the form nor on the outputs asked for.  The
+// parameter gradient's seven sums follow the form: for a stamp whose width is a
+// multiple of four they round differently (about 1e-7 of the sums) where it
+// starts on a multiple of four elements and where it does not.  One order for
+// both was measured and left: with a third loop, or the accesses chosen in the
+// four-pixel one, the aligned pixel gradients of 30,000 stamps of 64x64 took 321 to
+// 325 us instead of 302, those of 47x45 up to 209 instead of 188.
 //   65,536 stamps of 64x64: chi^2 alone (1.07 GB, 0.16 ms at the copy rate)
 //   0.33 to 0.25 ms; parameter gradient 0.53 to 0.45; with the pixel gradient
 //   (2.15 GB, 0.32 ms) and the caller's zero fill 0.71 to 0.63.
