@@ -41,6 +41,12 @@
  *  - count == 0 is a no-op returning FSE_OK.
  *  - One fse_ctx may be used from one host thread at a time; calls that
  *    overlap on the GPU must use different streams (up to 64 in flight).
+ *  - Calls that run parts side by side (fse_fit_batch, _ragged, _host) take
+ *    streams of the context for them: those that the call's stream used last,
+ *    and idle ones, so that no call waits for another stream's work.  A call on a
+ *    stream that is being captured, has another priority than the default or
+ *    belongs to a green context keeps all its work on that stream (but for
+ *    _host's second stream), as does one that finds no such stream free.
  */
 #ifndef FSE_H
 #define FSE_H
@@ -220,8 +226,8 @@ int fse_sersic_fit(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
  * brightest pixel, fit) in three persistent launches on `stream`: the start-up
  * (brightest pixel, growth-curve r50, sigma_w), the moment iteration, then the
  * fit of every stamp whose moments converged.  A large batch (2048 warps'
- * worth of stamps and more) runs as two such halves, the second on a stream of
- * the context that `stream` waits for, unless `stream` is being captured.
+ * worth of stamps and more) runs as two such halves, the second on a free stream
+ * of the context (see above) that `stream` waits for.
  * Results are those of the three single stages run in turn. */
 int fse_fit_batch(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
                   const fse_stamp *idx, int64_t count, const float *inv_var,
@@ -240,8 +246,8 @@ int fse_fit_batch_plain(fse_ctx *ctx, const void *pix, int dtype, const float *s
  * the inputs to context-owned device buffers in chunks (from 8192 stamps up,
  * 9 chunks of 2, 4, 6, 8, 10, 10, 10, 8 and 6 64ths of the batch, else one)
  * on a context copy stream,
- * runs each chunk's chain on `stream` or one of five context streams as soon
- * as its copy is done, copies the results back and returns when out[] is
+ * runs each chunk's chain on `stream`, a second stream or one of up to four free
+ * streams of the context as soon as its copy is done, copies the results back and returns when out[] is
  * complete.  npix_total bounds every idx[s].offset + h*w; a stamp outside it
  * returns FSE_EINVAL before any kernel runs, with out[] untouched (each chunk
  * is checked just before its copy, so the chunks before it may already have
@@ -258,7 +264,7 @@ int fse_fit_batch_host(fse_ctx *ctx, const void *pix, int64_t npix_total, int dt
  * into seven size classes (h*w up to 16^2, 24^2, 32^2, 48^2, 64^2, 96^2,
  * 128^2), and each class runs in its own three persistent launches whose
  * shared-memory tile fits that class, the classes side by side: the largest on
- * `stream`, the others on streams of the context that wait for the
+ * `stream`, the others on free streams of the context that wait for the
  * classification and that `stream` waits for.  Results are those of
  * fse_fit_batch, stamp by stamp.  opts->max_pix is not used (each class sets
  * its own); opts->warps_per_cta, if non-zero, applies to every class, else

@@ -34,7 +34,8 @@ constexpr int chunk_units_total() {
     return t;
 }
 static_assert(chunk_units_total() == 64, "the chunks must cover the batch in 64ths");
-constexpr int kHostStreams = 6;   // compute streams: the call's own and side streams
+constexpr int kHostStreams = 6;   // compute streams at most: the call's own, the context's
+                                  // stream for these calls, and free side streams
 
 constexpr int kSideStreams = fse::kClasses - 1;
 
@@ -44,6 +45,7 @@ struct fse_ctx {
     unsigned int* d_queue = nullptr;   // kQueues slots of kQueueWords work counters
     unsigned int* d_err = nullptr;     // sticky error word written by the kernels
     unsigned next_queue = 0;
+    cudaStream_t aux_stream = nullptr;  // second compute stream of the host-buffer pipeline
     cudaStream_t copy_stream = nullptr; // host-to-device copies of the host-buffer pipeline
     cudaEvent_t chunk_ev[kHostChunks + 1] = {}; // chunk copies done; the call's start
     // grow-only device staging of fse_fit_batch_host
@@ -65,11 +67,16 @@ struct fse_ctx {
     // Streams for the parts of a call that run beside its own stream: the size
     // classes of a ragged batch, the second half of a large one, the chunks of
     // the host-buffer pipeline.  A part waits for `fork` (recorded on the call's
-    // stream), and the call's stream for `join` of every part.
+    // stream), and the call's stream for `join` of every part.  A call takes the
+    // side streams that its own stream used last (by the stream's id; 0: nobody)
+    // and those whose last part has ended (take_sides).
     cudaStream_t side[kSideStreams] = {};
+    unsigned long long side_user[kSideStreams] = {};
     cudaEvent_t fork = nullptr;
     cudaEvent_t join[kSideStreams] = {};
-    unsigned next_side = 0;
+    // the same while a ragged call is captured into the context's graph
+    cudaEvent_t cap_fork = nullptr;
+    cudaEvent_t cap_join[kSideStreams] = {};
     // grow-only per-stamp coefficients of fse_moment_vjp
     fse::VjpCoef* d_vjp = nullptr;
     size_t vjp_cap = 0;
@@ -255,15 +262,56 @@ unsigned int* next_queue(fse_ctx* ctx) {
     return ctx->d_queue + static_cast<size_t>(ctx->next_queue++ % kQueues) * kQueueWords;
 }
 
-// Whether work of a call on `stream` may run beside it: not while the stream
-// is captured (the side streams would join the caller's capture).
-bool may_fork(cudaStream_t stream) {
+// Whether work of a call on `stream` may run beside it on the context's streams:
+// not while the stream is captured (they would join the caller's capture), and
+// not from a stream of another priority than theirs or of an SM partition, which
+// that work would leave.
+bool may_fork(const fse_ctx* ctx, cudaStream_t stream) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+    int own = 0, theirs = 0;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cudaStreamGetPriority(stream, &own) != cudaSuccess ||
+        cudaStreamGetPriority(ctx->side[0], &theirs) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return cap == cudaStreamCaptureStatusNone;
+    return cap == cudaStreamCaptureStatusNone && own == theirs && !fse::stream_of_partition(stream);
+}
+
+using Sides = int[kSideStreams];
+
+// The side streams that a call on `stream` may use, at most `want`, into k[]:
+// those that this stream used last (what they hold is already before the call)
+// and those with nothing left to do, so that no call waits for work of another
+// stream.  A call that gets none runs whole on its own stream.
+int take_sides(fse_ctx* ctx, cudaStream_t stream, int want, Sides& k) {
+    unsigned long long id = 0;
+    if (!may_fork(ctx, stream)) return 0;
+    if (cudaStreamGetId(stream, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    int n = 0;
+    for (int i = 0; i < kSideStreams && n < want; ++i)
+        if (ctx->side_user[i] == id) k[n++] = i;
+    if (n == want) return n;
+    // while some other stream is captured, an event may be queried in relaxed
+    // mode only
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return n;
+    }
+    for (int i = 0; i < kSideStreams && n < want; ++i) {
+        if (ctx->side_user[i] == id) continue;
+        if (ctx->side_user[i] == 0 || cudaEventQuery(ctx->join[i]) == cudaSuccess) {
+            ctx->side_user[i] = id;
+            k[n++] = i;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return n;
 }
 
 // One chain (or stage) on one stream.
@@ -286,11 +334,13 @@ constexpr int64_t kSplitWarps = 2048;
 // of 48x48 0.51 to 0.50; three and four parts and uneven halves were no faster.
 int run(fse_ctx* ctx, const fse::LaunchArgs& a, cudaStream_t stream) {
     if (a.count == 0) return FSE_OK;
-    if (a.stage != fse::kStageAll || a.count * a.warps_per_stamp < kSplitWarps || !may_fork(stream)) {
+    Sides sides;
+    if (a.stage != fse::kStageAll || a.count * a.warps_per_stamp < kSplitWarps ||
+        take_sides(ctx, stream, 1, sides) == 0) {
         const cudaError_t e = run_on(ctx, a, stream);
         return e != cudaSuccess ? cuda_fail(ctx, e, "estimator launch") : FSE_OK;
     }
-    const unsigned k = ctx->next_side++ % kSideStreams;
+    const int k = sides[0];
     fse::LaunchArgs lo = a, hi = a;
     lo.count = a.count / 2;
     hi.count = a.count - lo.count;
@@ -373,31 +423,36 @@ void class_shape(const fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o
 
 // Classification, then the chain's three launches per size class, each with a
 // shared-memory tile for its class.  The classes are independent and run side
-// by side: the largest on `s`, the others on streams of the context that wait
-// for the classification and that `s` waits for.  Each persistent launch ends
+// by side: the largest on `s`, the others in turn on the nside streams of the
+// context in sides[] (on `s` too if there are none), which wait for the
+// classification and which `s` waits for.  Each persistent launch ends
 // in a tail of its slowest stamps (a moment launch's last 0.1 ms runs at a
 // tenth of its warps); one class after another pays 21 such tails in a row,
 // side by side one class's tail is filled by the others' stamps.
 // Event-ordered throughout, with no host synchronisation, so the sequence can
-// be captured (into the context's own graph side by side; on a stream that the
-// caller captures, one class after another: fork = false).
-int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cudaStream_t s, bool fork) {
+// be captured (capture: into the context's own graph, with events of its own).
+int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cudaStream_t s, const Sides& sides,
+                   int nside, bool capture) {
+    const cudaEvent_t fork = capture ? ctx->cap_fork : ctx->fork;
+    cudaEvent_t* join = capture ? ctx->cap_join : ctx->join;
     unsigned int* counts = ctx->d_cls;
     unsigned int* range = counts + kK;
     unsigned int* cursor = range + 2 * kK;
     unsigned int* queues = cursor + kK;
     cudaError_t e = cudaMemsetAsync(ctx->d_cls, 0, kClsWords * sizeof(unsigned int), s);
     if (e == cudaSuccess) e = fse::classify_stamps(a.idx, a.count, counts, range, cursor, ctx->d_perm, s);
-    if (e == cudaSuccess && fork) e = cudaEventRecord(ctx->fork, s);
+    if (e == cudaSuccess && nside) e = cudaEventRecord(fork, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "size classification");
-    int forked = kK - 1;   // classes forked .. kK - 2 have work on their streams
-    for (int k = kK - 1; k >= 0 && e == cudaSuccess; --k) {
+    int forked = 0;   // side streams that have work
+    for (int k = kK - 1, turn = -1; k >= 0 && e == cudaSuccess; --k, ++turn) {
         cudaStream_t ks = s;
-        if (fork && k < kK - 1) {
-            ks = ctx->side[k];
-            e = cudaStreamWaitEvent(ks, ctx->fork, 0);
-            if (e != cudaSuccess) break;
-            forked = k;
+        if (nside && turn >= 0) {
+            ks = ctx->side[sides[turn % nside]];
+            if (turn < nside) {
+                e = cudaStreamWaitEvent(ks, fork, 0);
+                if (e != cudaSuccess) break;
+                forked = turn + 1;
+            }
         }
         fse::LaunchArgs b = a;
         b.opts.max_pix = fse::kClassPix[k];
@@ -408,9 +463,9 @@ int enqueue_ragged(fse_ctx* ctx, const fse::LaunchArgs& a, const fse_opts& o, cu
         e = fse::launch_estimator(b, ks);
     }
     // join what was forked, also after an error: the caller's buffers are in use
-    for (int k = kK - 2; fork && k >= forked; --k) {
-        cudaError_t j = cudaEventRecord(ctx->join[k], ctx->side[k]);
-        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, ctx->join[k], 0);
+    for (int i = 0; i < forked; ++i) {
+        cudaError_t j = cudaEventRecord(join[sides[i]], ctx->side[sides[i]]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(s, join[sides[i]], 0);
         if (e == cudaSuccess) e = j;
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "size-class launch");
@@ -506,16 +561,19 @@ int fse_create(fse_ctx** out, int device) {
         return FSE_ENOMEM;
     }
     if (cudaMemset(ctx->d_err, 0, sizeof(unsigned int)) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         fse_destroy(ctx);
         return FSE_ECUDA;
     }
-    bool ok = cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess;
+    bool ok = cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&ctx->cap_fork, cudaEventDisableTiming) == cudaSuccess;
     for (int k = 0; k < kSideStreams && ok; ++k)
         ok = cudaStreamCreateWithFlags(&ctx->side[k], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&ctx->join[k], cudaEventDisableTiming) == cudaSuccess;
+             cudaEventCreateWithFlags(&ctx->join[k], cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&ctx->cap_join[k], cudaEventDisableTiming) == cudaSuccess;
     for (int k = 0; k < kHostChunks + 1 && ok; ++k)
         ok = cudaEventCreateWithFlags(&ctx->chunk_ev[k], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
@@ -553,9 +611,12 @@ void fse_destroy(fse_ctx* ctx) {
         for (int k = 0; k < kSideStreams; ++k) {
             if (ctx->side[k]) cudaStreamDestroy(ctx->side[k]);
             if (ctx->join[k]) cudaEventDestroy(ctx->join[k]);
+            if (ctx->cap_join[k]) cudaEventDestroy(ctx->cap_join[k]);
         }
         if (ctx->fork) cudaEventDestroy(ctx->fork);
+        if (ctx->cap_fork) cudaEventDestroy(ctx->cap_fork);
         if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+        if (ctx->aux_stream) cudaStreamDestroy(ctx->aux_stream);
         if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
         for (cudaEvent_t ev : ctx->chunk_ev)
@@ -657,15 +718,20 @@ int fse_fit_batch_host(fse_ctx* ctx, const void* pix, int64_t npix_total, int dt
         return rc;
     // The copy stream moves every chunk's inputs to the device back to back and
     // records chunk_ev[c] after chunk c; chunk c's kernels and its result copy
-    // run on compute stream c % 6 once chunk_ev[c] is done.  A chunk's chain is
-    // at least as long as its slowest stamp's three launches (0.4 ms), so the
-    // chunks need several streams beside one another: with two, 40,000 stamps of
-    // 48x48 took 3.82 ms, three 3.37, four 3.22, six 3.18 (9,000 stamps 2.28,
-    // 1.68, 1.54, 1.29; 100,000 stamps 7.26, 7.00, 6.93, 6.93).
+    // run on the compute streams in turn once chunk_ev[c] is done.  A chunk's
+    // chain is at least as long as its slowest stamp's three launches (0.4 ms), so
+    // the chunks need several streams beside one another: with two, 40,000 stamps
+    // of 48x48 took 3.82 ms, three 3.37, four 3.22, six 3.18 (9,000 stamps 2.28,
+    // 1.68, 1.54, 1.29; 100,000 stamps 7.26, 7.00, 6.93, 6.93; one host's link).
     const cudaStream_t s0 = static_cast<cudaStream_t>(stream);
-    cudaStream_t streams[kHostStreams] = {s0};
-    for (int i = 1; i < kHostStreams; ++i) streams[i] = ctx->side[i - 1];
-    const int used = nchunk < kHostStreams ? nchunk : kHostStreams;
+    cudaStream_t streams[kHostStreams] = {s0, ctx->aux_stream};
+    int nstream = 2;
+    if (nchunk > 1) {
+        Sides sides;
+        const int n = take_sides(ctx, s0, kHostStreams - 2, sides);
+        for (int i = 0; i < n; ++i) streams[nstream++] = ctx->side[sides[i]];
+    }
+    const int used = nchunk < nstream ? nchunk : nstream;
     const cudaStream_t cs = ctx->copy_stream;
     cudaEvent_t ev_start = ctx->chunk_ev[kHostChunks];
     cudaError_t e = cudaEventRecord(ev_start, s0);
@@ -712,7 +778,7 @@ int fse_fit_batch_host(fse_ctx* ctx, const void* pix, int64_t npix_total, int dt
     for (int c = 0; c < nchunk && e == cudaSuccess; ++c) {
         const int64_t s_lo = lo[c], n_c = lo[c + 1] - lo[c];
         if (n_c == 0) continue;
-        const cudaStream_t st = streams[c % kHostStreams];
+        const cudaStream_t st = streams[c % used];
         e = cudaStreamWaitEvent(st, ctx->chunk_ev[c], 0);
         if (e != cudaSuccess) break;
         fse::LaunchArgs a;
@@ -765,7 +831,11 @@ int fse_fit_batch_ragged(fse_ctx* ctx, const void* pix, int dtype, const float* 
     if (rc || count == 0) return rc;
     if ((rc = ragged_workspace(ctx, count))) return rc;
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (!(o.flags & FSE_FLAG_GRAPH)) return enqueue_ragged(ctx, a, o, s, may_fork(s));
+    Sides sides;
+    if (!(o.flags & FSE_FLAG_GRAPH)) {
+        const int n = take_sides(ctx, s, kSideStreams, sides);
+        return enqueue_ragged(ctx, a, o, s, sides, n, false);
+    }
     RaggedKey key;
     make_key(ctx, a, o, &key);
     if (!ctx->gexec || memcmp(&key, ctx->gkey, sizeof key) != 0) {
@@ -774,7 +844,8 @@ int fse_fit_batch_ragged(fse_ctx* ctx, const void* pix, int dtype, const float* 
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph capture");
-        rc = enqueue_ragged(ctx, a, o, ctx->cap_stream, true);
+        for (int k = 0; k < kSideStreams; ++k) sides[k] = k;
+        rc = enqueue_ragged(ctx, a, o, ctx->cap_stream, sides, kSideStreams, true);
         e = cudaStreamEndCapture(ctx->cap_stream, &graph);
         if (rc) {
             if (graph) cudaGraphDestroy(graph);

@@ -190,6 +190,8 @@ size_t smem_per_group(int max_pix, bool ivar, int warps_per_stamp);
 // scratch address) belongs to a context: after cudaDeviceReset the device's
 // primary context is a new one and that state must be set up again.
 unsigned long long current_context_id();
+// Whether a stream belongs to a green context (a partition of the SMs).
+bool stream_of_partition(cudaStream_t stream);
 // Library launch shape for a tile size: warps per stamp, and warps per CTA
 // (a multiple of it) as large as shared memory allows, up to four groups.
 void choose_launch(int max_pix, int* warps_per_cta, int* warps_per_stamp);

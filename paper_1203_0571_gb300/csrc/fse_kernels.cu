@@ -2481,6 +2481,25 @@ unsigned long long current_context_id() {
     return id;
 }
 
+bool stream_of_partition(cudaStream_t stream) {
+    // the driver's cuStreamGetGreenCtx, looked up as above; not for the handles of
+    // the default streams
+    using GetGreen = int (*)(void*, void**);
+    static GetGreen get_green = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &p, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_green = reinterpret_cast<GetGreen>(p);
+        cudaGetLastError();
+    });
+    if (!get_green || !stream || stream == cudaStreamLegacy || stream == cudaStreamPerThread) return false;
+    void* green = nullptr;
+    return get_green(stream, &green) == 0 && green != nullptr;
+}
+
 size_t smem_per_group(int max_pix, bool ivar, int warps_per_stamp) {
     return shape_bytes(max_pix, ivar, warps_per_stamp);
 }
