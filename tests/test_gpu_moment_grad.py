@@ -269,3 +269,44 @@ def test_moment_grad_edge_cases(ctx):
             ctx.moment_vjp(b.pix, idx, moments, v, mode=bad)
     # an empty batch is a no-op
     ctx.moment_jvp(b.pix, idx[:0], moments[:0], torch.zeros(0, device="cuda"))
+
+
+@pytest.mark.parametrize("h,w", [(48, 48), (45, 47)])
+def test_tangents_far_from_the_weight(ctx, h, w):
+    """A tangent of one pixel where the weight is below 2^-40 moves the shape by
+    what the VJP gives for that pixel: the Jacobian and its transpose run over
+    the same pixels.  Both form W = 2^x from x = -R^2 log2(e) / 2 s^2 in fp32, here
+    -100 < x < -41, with a few roundings of terms up to |x| each (below 1e-4 of
+    W); 1e-3 leaves room for the solve."""
+    img = synth.single_stamp(h, w, n=0.5, re=2.0, g1=0.1, g2=-0.05, xc=w / 2 - 0.3, yc=h / 2 + 0.2, I0=300.0,
+                             noise_sigma=0.3, seed=3)
+    n = 6
+    batch = synth.StampBatch(pix=torch.as_tensor(np.tile(img.astype(np.float32).ravel(), n)),
+                             offset=torch.arange(n) * h * w, h=torch.full((n,), h, dtype=torch.int32),
+                             w=torch.full((n,), w, dtype=torch.int32), truth={})
+    b = batch.to("cuda")
+    idx = B.make_index(b.offset, b.h, b.w)
+    opts = B.default_opts(max_pix=h * w)
+    mom = ctx.centroid(b.pix, idx, opts=opts)
+    ctx.ellipticity(b.pix, idx, mom, opts=opts)
+    r = B.results(mom)[0]
+    yy, xx = np.mgrid[0:h, 0:w]
+    t1, t2, g1, g2 = xx - r["x0"], yy - r["y0"], r["e1"], r["e2"]
+    R2 = ((1 - g1) ** 2 + g2 ** 2) * t1 ** 2 + ((1 + g1) ** 2 + g2 ** 2) * t2 ** 2 - 4 * g2 * t1 * t2
+    x = -R2 * 1.4426950408889634 / (2 * r["sigma_w"] ** 2)
+    far = np.argwhere((x < -41) & (x > -100))
+    # above and below the weight's rows, and beside them
+    pick = [far[0], far[-1], far[np.argmin(np.abs(far[:, 0] - r["y0"]))]] * 2
+    tan = np.zeros((n, h, w), np.float32)
+    for i, (pr, pc) in enumerate(pick):
+        tan[i, pr, pc] = 2.0 ** 60
+    mode = B.FSE_MOM_ELLIP | B.FSE_MOM_SIGW_FIXED
+    jvp = ctx.moment_jvp(b.pix, idx, mom, torch.as_tensor(tan.ravel()).cuda(), mode=mode).cpu().numpy()
+    for k in range(4):
+        v = torch.zeros((n, 5), device="cuda")
+        v[:, k] = 1.0
+        dp = ctx.moment_vjp(b.pix, idx, mom, v, mode=mode).cpu().numpy().reshape(n, h, w)
+        for i, (pr, pc) in enumerate(pick):
+            want = float(dp[i, pr, pc]) * 2.0 ** 60
+            scale = max(abs(float(dp[i, pr, pc])), 1e-3 * float(np.abs(dp[i, pr]).max())) * 2.0 ** 60
+            assert want != 0 and abs(jvp[i, k] - want) <= 1e-3 * scale, (k, i, jvp[i, k], want)
