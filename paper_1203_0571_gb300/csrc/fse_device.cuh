@@ -335,7 +335,9 @@ struct FWalk {
 // A t1^2 + B t2^2 - 4 g2 t1 t2 <= Rc^2 (Eq. A1; the determinant of the form
 // is (1 - |g|^2)^2) lies inside |t1| <= Rc sqrt(B) / (1 - |g|^2), |t2| <=
 // Rc sqrt(A) / (1 - |g|^2); the box adds a pixel of margin and is cut to the
-// stamp.  Compact objects (stars, small galaxies) cover a fraction of their
+// stamp (2^15 px is past any: the gradients take strips of up to FSE_MAX_PIX
+// pixels).  (A record with |g| > 1 gets the whole stamp, or a box of the centre's
+// neighbours where the ellipse is narrower than that.)  Compact objects (stars, small galaxies) cover a fraction of their
 // stamp, which is the work saved.
 constexpr float kWeightCut = 7.4446500f;   // sqrt(80 ln 2)
 
@@ -346,11 +348,11 @@ struct Box {
     __device__ __forceinline__ int last(int w) const { return (r0 + bh - 1) * w + c0 + bw - 1; }
 };
 
-__device__ __forceinline__ Box weight_box(float xc, float yc, float g1, float g2, float sw, int h, int w) {
+__host__ __device__ __forceinline__ Box weight_box(float xc, float yc, float g1, float g2, float sw, int h, int w) {
     const float gg = g1 * g1 + g2 * g2;
     const float rc = kWeightCut * sw / (1.f - gg);
-    const float hx = fminf(rc * sqrtf(1.f + gg + 2.f * g1) + 1.f, 4096.f);
-    const float hy = fminf(rc * sqrtf(1.f + gg - 2.f * g1) + 1.f, 4096.f);
+    const float hx = fminf(rc * sqrtf(1.f + gg + 2.f * g1) + 1.f, 32768.f);
+    const float hy = fminf(rc * sqrtf(1.f + gg - 2.f * g1) + 1.f, 32768.f);
     Box b;
     b.c0 = max(0, static_cast<int>(floorf(xc - hx)));
     b.r0 = max(0, static_cast<int>(floorf(yc - hy)));
@@ -369,10 +371,10 @@ __device__ __forceinline__ Box weight_box(float xc, float yc, float g1, float g2
     return b;
 }
 
-// a / b for 0 <= a <= 256 and 1 <= b <= 128, from ib = 1 / b to a few ulps:
-// (a + 1/2) / b lies at least 1/256 from every integer, and the product is off
-// by less than 1e-4.
-__device__ __forceinline__ int div_small(int a, float ib) {
+// a / b for 0 <= a <= 256 and 1 <= b, from ib = 1 / b to a few ulps: for b <= 256
+// (a + 1/2) / b lies at least 1/512 from every integer, and the product is off by
+// less than 1e-4; above, both are below 1.
+__host__ __device__ __forceinline__ int div_small(int a, float ib) {
     return static_cast<int>((static_cast<float>(a) + 0.5f) * ib);
 }
 
