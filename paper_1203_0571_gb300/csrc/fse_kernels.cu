@@ -2348,12 +2348,13 @@ cudaError_t launch_t(const LaunchArgs& a_in, cudaStream_t stream) {
     int groups = a.warps_per_cta / NW;
     if (groups < 1 || groups * NW != a.warps_per_cta || groups > 15) return cudaErrorInvalidValue;
     const size_t spg = stage_group_bytes(STAGE, a.opts.max_pix, DT == FSE_BF16, IVAR, NW, a.opts.ring_slots);
+    // what a fit shape may take is stated by shape_bytes, with any model
+    if (STAGE == kStageFit && shape_bytes(a.opts.max_pix, IVAR, NW) * groups > 227 * 1024) return cudaErrorInvalidValue;
     if constexpr (STAGE == kStageFit && !SUP) {
         // Tensor memory is allocated in columns over all four quadrants, so a
         // CTA of fewer than four warps would leave the other quadrants' lanes
         // idle: such a shape is widened to four warps as far as shared memory
         // allows (groups are independent; the results do not depend on it).
-        if (shape_bytes(a.opts.max_pix, IVAR, NW) * groups > 227 * 1024) return cudaErrorInvalidValue;
         if (!a.static_assign)
             while (groups * NW < 4 && spg * (2 * groups) <= 226 * 1024) groups *= 2;
         a.warps_per_cta = groups * NW;

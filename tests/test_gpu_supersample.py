@@ -152,3 +152,22 @@ def test_supersample_options(ctx):
     a = B.results(ctx.fit_batch(batch.pix, idx, opts=B.default_opts(max_pix=1024, supersample=0)))
     c = B.results(ctx.fit_batch(batch.pix, idx, opts=B.default_opts(max_pix=1024)))
     assert a.tobytes() == c.tobytes()
+
+
+def test_shapes_that_do_not_fit_are_refused(ctx):
+    """Launch shapes are accepted by the tile that the library states for them
+    (two floats a pixel, three with weights), with the pixel-integrated model as
+    without it: eight warps of 64x64 tiles do not fit an SM."""
+    batch = synth.make_workload(0, count=8).to("cuda")
+    idx = B.make_index(batch.offset, batch.h, batch.w)
+    mom = ctx.centroid(batch.pix, idx, opts=B.default_opts(max_pix=1024))
+    ctx.ellipticity(batch.pix, idx, mom, opts=B.default_opts(max_pix=1024))
+    for ss in (1, 2):
+        for warps, fits in ((4, True), (8, False)):
+            opts = B.default_opts(max_pix=64 * 64, supersample=ss, warps_per_cta=warps)
+            if fits:
+                ctx.sersic_fit(batch.pix, idx, mom.clone(), opts=opts)
+            else:
+                with pytest.raises(B.FseError):
+                    ctx.sersic_fit(batch.pix, idx, mom.clone(), opts=opts)
+    ctx.sync_check()
