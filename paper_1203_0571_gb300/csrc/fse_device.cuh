@@ -214,9 +214,9 @@ __device__ __forceinline__ FixScale fix_scale(float amax, int npix, int b) {
     f.up2 = ldexpf(1.f, S - 2 * f.B);
     f.dn2 = -ldexpf(1.f, 2 * f.B - S);
     f.dn1 = -ldexpf(1.f, f.B - S);
-    // |q2| <= 2^(62 - 2b) / npix has to be below 2^22 (the rounding add), or the
+    // |q2| <= 2^(62 - 2b) / npix has to be at most 2^22 (the rounding add), or the
     // 64-bit conversion is taken; so too where the scale itself overflows
-    f.wide = !(top < INFINITY) || (static_cast<long long>(npix) << (2 * b)) < (1ll << 40);
+    f.wide = !(top < INFINITY) || (b < 20 && npix < 1 << (40 - 2 * b));
     return f;
 }
 

@@ -228,3 +228,30 @@ def test_cutout_total_of_saturated_values(ctx):
     assert torch.equal(res[0], res[1]), [r.view(torch.float32)[0, 4] for r in res]
     r50 = float(res[0].view(torch.float32)[0, 4])
     assert abs(r50 - (side * side / (2 * np.pi)) ** 0.5) < 1.0, r50
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_cutout_of_large_images(ctx, O, dtype):
+    """Images of 2^19 pixels and more, whose values need two fixed-point pieces;
+    with a side above 2048 the general ring index."""
+    rng = np.random.default_rng(12)
+    pix, offs, hs, ws, pos = [], [], [], [], 0
+    for h, w in [(725, 724), (1100, 1001), (2100, 300)]:
+        yy, xx = np.mgrid[0:h, 0:w].astype(np.float64)
+        for r50 in (4.0, 90.0):
+            s = r50 / 1.1774
+            I = 100.0 * np.exp(-((xx - w / 2 + 0.2) ** 2 + (yy - h / 2 - 0.3) ** 2) / (2 * s * s))
+            pix.append((I + rng.normal(0, 0.002, (h, w))).astype(np.float32).ravel())
+            offs.append(pos)
+            hs.append(h)
+            ws.append(w)
+            pos += h * w
+    batch = synth.StampBatch(pix=torch.as_tensor(np.concatenate(pix)), offset=torch.as_tensor(offs),
+                             h=torch.as_tensor(hs, dtype=torch.int32), w=torch.as_tensor(ws, dtype=torch.int32),
+                             truth={})
+    if dtype == "bf16":
+        batch = synth.encode_bf16(batch)
+    batch = batch.to("cuda")
+    out, cidx, info = ctx.cutout(batch.pix, B.make_index(batch.offset, batch.h, batch.w), scale=batch.scale)
+    torch.cuda.synchronize()
+    check_against_oracle(O, batch, out, cidx, info)
