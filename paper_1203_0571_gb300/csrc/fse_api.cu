@@ -22,10 +22,12 @@
 // and shrink again so that little compute is left once the last copy is done.
 // The host link's rate differs between machines (211 GB/s measured on one
 // GB300 host; another behaved as about 120 GB/s, against about 100 GB/s of
-// pixels consumed by the kernels on 48x48 stamps), and by a model of the
-// pipeline this schedule stays within 10% of the best over that range; few chunks, because every chunk adds two launch tails
-// (on 100,000 stamps of 48x48, twelve chunks cost 11.0 ms against 9.5 ms for
-// one launch pair).
+// pixels consumed by an earlier build's kernels on 48x48 stamps, 170 by today's),
+// and by a model of the pipeline this schedule stayed within 10% of the best over
+// that range with that build, whose chunks ran on two streams: every chunk adds its
+// launches' tails (100,000 stamps of 48x48 in twelve chunks 11.0 ms against 9.5 ms
+// of kernels).  With six streams the tails overlap; the schedule was not measured
+// again with them.
 constexpr int kHostChunks = 9;
 constexpr int kChunkUnits[kHostChunks] = {2, 4, 6, 8, 10, 10, 10, 8, 6};
 constexpr int chunk_units_total() {
@@ -329,9 +331,10 @@ constexpr int64_t kSplitWarps = 2048;
 // The whole chain of a large batch runs as two halves, the second on a side
 // stream: each of the chain's three launches ends in a tail of its slowest
 // stamps (0.45 ms a call on one stream, whatever its size), and the other
-// half's launches fill it.  Results do not depend on it.  100,000 stamps of
-// 48x48 5.86 to 5.68 ms, 20,000 1.54 to 1.39, 8,000 of 64x64 1.25 to 1.11, 3,000
-// of 48x48 0.51 to 0.50; three and four parts and uneven halves were no faster.
+// half's launches fill it.  Results do not depend on it.  When it came in:
+// 100,000 stamps of 48x48 5.86 to 5.68 ms, 20,000 1.54 to 1.39, 8,000 of 64x64 1.25
+// to 1.11, 3,000 of 48x48 0.51 to 0.50; three and four parts and uneven halves were
+// no faster.
 int run(fse_ctx* ctx, const fse::LaunchArgs& a, cudaStream_t stream) {
     if (a.count == 0) return FSE_OK;
     Sides sides;

@@ -127,10 +127,10 @@ __device__ __forceinline__ float max_abs_nan(float a, float b) {
 // shared memory and is combined in the same order in each of them, so they
 // hold the same values and take the same branches.
 //   500 images of 512x512 fp32 (524 MB, 0.077 ms at the copy rate), whole call:
-//   0.866 ms with every pixel binned (152 instructions a pixel), 0.225 ms with
-//   the square.  What is left: 0.07 ms for the first pass (DRAM), 0.02 for the
-//   second, the images that need every ring (a tenth; 0.03), and the cluster
-//   barriers and starts; clusters of four took 0.25 ms, five CTAs per SM 0.24.
+//   0.85 ms with every pixel binned (152 instructions a pixel), 0.20 ms with the
+//   square.  What is left: 0.07 ms for the first pass (DRAM), 0.02 for the second,
+//   the images that need every ring (a tenth; 0.03), and the cluster barriers and
+//   starts; clusters of four cost 0.03 ms more, five CTAs per SM 0.02.
 constexpr int kNear = 24;                 // half-side of the square, and its last ring
 constexpr int kFixBits = 22;              // piece width of the total and the near rings (at
                                           // most 200 pixels each)

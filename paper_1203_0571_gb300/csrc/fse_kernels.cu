@@ -2319,7 +2319,7 @@ __global__ void __maxnreg__(moment_stage(STAGE) ? (NW >= 8 ? 128 : 96) : (SUP ? 
                 res.flux = st.yf;
             }
         }
-        if (!skip && (STAGE == kStageFit || STAGE == kStageAll)) {
+        if (!skip && STAGE == kStageFit) {
             const FitOut f = sersic_fit<IVAR, NW, SUP>(s, tm, ivbuf, qmax, h, w, npix, g, o, st, status);
             res.I0 = static_cast<float>(f.I0);
             res.re = static_cast<float>(f.re);
