@@ -368,9 +368,9 @@ int fse_star_fit(fse_ctx *ctx, const void *pix, int dtype, const float *scale,
  * FSE_ST_NONFINITE, FSE_ST_BAD_SIZE (h*w above FSE_MAX_PIX: nothing written),
  * FSE_ST_FIT_SINGULAR (J singular); such stamps get zero derivatives.
  * bf16 pixels are decoded with scale[s]; the derivatives are with respect to
- * the decoded intensities.  J is summed over the rows where the weight reaches
- * 2^-40 (the moment stage's own cut); the tangent, and dL/dI, over every pixel.
- * Device pointers; asynchronous on `stream`.  The VJP runs two launches: one for the sums, J and the solve (96 bytes of
+ * the decoded intensities.  The VJP sums J over the rows where the weight
+ * reaches 2^-40 (the moment stage's own cut) and writes every pixel; the JVP's
+ * sums take every pixel.  Device pointers; asynchronous on `stream`.  The VJP runs two launches: one for the sums, J and the solve (96 bytes of
  * coefficients per stamp), then one that writes dL/dI from them.  The
  * coefficients live in a grow-only scratch buffer of the context, allocated,
  * with a device synchronisation, when a call has more stamps than any before

@@ -315,30 +315,14 @@ __device__ R50Grad r50_ring(const MomentGradArgs& a, const fse_stamp& ix, float 
     return o;
 }
 
-// The weight at t = (t1, t2).
-__device__ __forceinline__ float weight(const Geom& q, float t1, float t2) {
-    return ex2(fmaf(q.A, t1 * t1, fmaf(q.B, t2 * t2, -q.G4 * (t1 * t2))) * q.cw);
-}
-
-// The JVP's terms of one pixel: the tangent u W times the six monomials of
-// degree <= 2 into PU.
-__device__ __forceinline__ void tangent_terms(float W, float t1, float t2, float uu, float (&PU)[6]) {
-    const float h = uu * W;
-    const float h1 = h * t1, h2 = h * t2;
-    PU[0] += h;
-    PU[1] += h1;
-    PU[2] += h2;
-    PU[3] = fmaf(h1, t1, PU[3]);
-    PU[4] = fmaf(h1, t2, PU[4]);
-    PU[5] = fmaf(h2, t2, PU[5]);
-}
-
 // The moment terms of one pixel at t = (t1, t2): f = I W times the 15
-// monomials of degree <= 4 into P; for the JVP, the tangent's into PU.
+// monomials of degree <= 4 into P; for the JVP, the tangent u W times the
+// six of degree <= 2 into PU.
 template <bool JVP>
 __device__ __forceinline__ void moment_terms(const Geom& q, float t1, float t2, float v, float uu, float (&P)[15],
                                              float (&PU)[6]) {
-    const float W = weight(q, t1, t2);
+    const float R2 = fmaf(q.A, t1 * t1, fmaf(q.B, t2 * t2, -q.G4 * (t1 * t2)));
+    const float W = ex2(R2 * q.cw);
     const float f = v * W;
     const float f1 = f * t1, f2 = f * t2;
     const float f11 = f1 * t1, f12 = f1 * t2, f22 = f2 * t2;
@@ -358,20 +342,31 @@ __device__ __forceinline__ void moment_terms(const Geom& q, float t1, float t2, 
     P[mono(2, 2)] = fmaf(f112, t2, P[mono(2, 2)]);
     P[mono(1, 3)] = fmaf(f122, t2, P[mono(1, 3)]);
     P[mono(0, 4)] = fmaf(f222, t2, P[mono(0, 4)]);
-    if (JVP) tangent_terms(W, t1, t2, uu, PU);
+    if (JVP) {
+        const float h = uu * W;
+        const float h1 = h * t1, h2 = h * t2;
+        PU[0] += h;
+        PU[1] += h1;
+        PU[2] += h2;
+        PU[3] = fmaf(h1, t1, PU[3]);
+        PU[4] = fmaf(h1, t2, PU[4]);
+        PU[5] = fmaf(h2, t2, PU[5]);
+    }
 }
 
 // The weighted sums of one stamp, by one warp, in one pass over its pixels
 // (eight loads in flight per lane): finiteness; with sigma_w from the growth
-// curve the brightest pixel and the total; for the JVP the tangent's total and
-// its six weighted moments, of every pixel (a tangent may be all where the
-// weight is small, and the VJP writes every pixel); and, where the rows of a block
-// of 256 pixels meet the weight's box (W >= 2^-40, weight_box; the rest adds less
-// than 2^-40 |I| |t|^4 to a sum, the iteration's own cut), the 15 weighted moments:
-// eight pixels per lane in fp32, then double-float.  Then the growth curve's
-// crossing ring (r50_ring).  The totals go to rec from the lanes that hold them
-// after the exchange.  (A second pass over the box's pixels alone has a third
-// fewer weights to evaluate, but its walk and its wait for the loads cost more.)
+// curve the brightest pixel and the total; the 15 weighted moments; and for the
+// JVP the tangent's total and its six: eight pixels per lane in fp32, then
+// double-float.  The VJP leaves out blocks of 256 pixels whose rows do not meet the
+// weight's box (W >= 2^-40, weight_box; they add less than 2^-40 |I| |t|^4 to a sum,
+// the iteration's own cut).  The JVP takes every block: a tangent may be all where
+// the weight is small, as the VJP writes every pixel; and 20,000 stamps of 48x48
+// take 217 us, with the tangent alone summed outside the box 247, with both cut to
+// it 225 (64x64 316, 337, 295).  Then the growth curve's crossing ring (r50_ring).
+// The totals go to rec from the lanes that hold them after the exchange.  (A
+// second pass over the box's pixels alone has a third fewer weights to evaluate,
+// but its walk and its wait for the loads cost more.)
 template <int DT, bool JVP>
 __device__ __forceinline__ void stamp_grad(const MomentGradArgs& a, int64_t si, int lane, MomSums* rec) {
     const fse_stamp ix = a.idx[si];
@@ -443,26 +438,16 @@ __device__ __forceinline__ void stamp_grad(const MomentGradArgs& a, int64_t si, 
                     df_add(th[0], tl[0], pt);
                 }
                 if (JVP) df_add(th[1], tl[1], pu);
-                float P[15], PU[6];
+                if (!JVP && (b0 + 256 <= box0 || b0 >= box1)) {
 #pragma unroll
-                for (int i = 0; i < 6; ++i) PU[i] = 0.f;
-                if (b0 + 256 <= box0 || b0 >= box1) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (JVP) {
-                            const float t1 = pw.c - q.x0, t2 = pw.r - q.y0;
-                            tangent_terms(weight(q, t1, t2), t1, t2, uu[u], PU);
-                        }
-                        pw.next();
-                    }
-                    if (JVP) {
-#pragma unroll
-                        for (int i = 0; i < 6; ++i) df_add(Uh[i], Ul[i], PU[i]);
-                    }
+                    for (int u = 0; u < 8; ++u) pw.next();
                     continue;
                 }
+                float P[15], PU[6];
 #pragma unroll
                 for (int i = 0; i < 15; ++i) P[i] = 0.f;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) PU[i] = 0.f;
                 // (pixels past the end are zero and add nothing)
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -599,10 +584,9 @@ __device__ __forceinline__ void stamp_grad(const MomentGradArgs& a, int64_t si, 
 
 // One warp per stamp, from the work counter.
 //   50,000 stamps of 48x48 (JVP, sigma_w from the growth curve; 922 MB read,
-//   0.136 ms at the copy rate): 0.87 ms with the ring's disc sums over the whole
+//   0.136 ms at the copy rate): 0.85 ms with the ring's disc sums over the whole
 //   stamp, a generic 42-term entry of J per lane and the 5 x 5 solve repeated in
-//   every lane; 0.73 ms with the warp sums by exchange; 0.54 ms as it is but for the
-//   tangent's sums of the box's rows only, 0.62 ms with those of every pixel, bound by
+//   every lane; 0.73 ms with the warp sums by exchange; 0.53 ms as it is, bound by
 //   issue and instruction fetch (2,000 instructions outside the pixel loop).  A
 //   lane per stamp for the solve, 32 stamps at a time, took 0.42 ms here but 75
 //   instead of 53 us at 2,090 stamps of 62x62, where it fetches its code for one
