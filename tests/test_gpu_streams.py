@@ -97,3 +97,31 @@ def test_kernels_keep_to_the_streams_priority(ctx, kind, tmp_path):
     high, plain = torch.cuda.Stream(priority=-1), torch.cuda.Stream()
     assert len(streams_of(lambda: f(b.pix, idx, opts=opts, out=out, stream=plain), tmp_path)) > 1
     assert len(streams_of(lambda: f(b.pix, idx, opts=opts, out=out, stream=high), tmp_path)) == 1
+
+
+def test_call_beside_a_capture(ctx):
+    """A call on one stream while the same thread captures another in global
+    mode, with the context's side streams in use elsewhere: the capture goes on,
+    and the call runs."""
+    batch, b, idx, opts = large()
+    want = ctx.fit_batch(b.pix, idx, opts=opts)
+    outs = [torch.zeros_like(want) for _ in range(2)]
+    x = torch.zeros(16, device="cuda")
+    sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+    for o, s in zip(outs, (sa, sb)):
+        ctx.fit_batch(b.pix, idx, opts=opts, out=o, stream=s)
+    torch.cuda.synchronize()
+    outs[1].zero_()
+    with torch.cuda.stream(sa):
+        torch.cuda._sleep(200_000_000)
+        ctx.fit_batch(b.pix, idx, opts=opts, out=outs[0], stream=sa)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        x += 1
+        ctx.fit_batch(b.pix, idx, opts=opts, out=outs[1], stream=sb)
+        x += 1
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], want) and torch.equal(outs[1], want)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x[0]) == 2.0
